@@ -244,6 +244,7 @@ extern "C" int tmd_create(const tmd_config* cfg, tmd_handle** out) {
       (rc = tmd_cuda_check(h, cudaEventCreateWithFlags(&h->scratch_done, cudaEventDisableTiming),
                            "event")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_count_rank(), "smem attribute")) != TMD_OK ||
+      (rc = tmd_cuda_check(h, prepare_unatt_encode(&h->occ_ue), "unattached encoder")) != TMD_OK ||
       (rc = tmd_cuda_check(h, occupancy_track_decode(0, &h->occ_decode_v[0]), "occupancy")) != TMD_OK ||
       (rc = tmd_cuda_check(h, occupancy_track_decode(1, &h->occ_decode_v[1]), "occupancy")) != TMD_OK ||
       (rc = tmd_cuda_check(h, occupancy_unatt_decode(&h->occ_unatt), "occupancy")) != TMD_OK ||
@@ -258,6 +259,7 @@ extern "C" int tmd_create(const tmd_config* cfg, tmd_handle** out) {
   if (!h->autotune_cache.empty()) tmd_tune_load(h);
   if (h->occ_unatt < 1) h->occ_unatt = 1;
   if (h->occ_encode < 1) h->occ_encode = 1;
+  if (h->occ_ue < 1) h->occ_ue = 1;
   *out = h;
   return TMD_OK;
 }

@@ -152,6 +152,9 @@ __global__ void k_track_scan2(const FrameDev* frames, PlanDev plan);
 // (grid: ranking tiles of all frames).
 void launch_count_rank(uint32_t grid, cudaStream_t st, const FrameDev* frames, PlanDev plan);
 cudaError_t prepare_count_rank();
+// Shared-memory attributes of the unattached encoder; resident blocks per SM
+// of its cooperative kernel.
+cudaError_t prepare_unatt_encode(int* blocks_per_sm);
 __global__ void k_group_sum(const FrameDev* frames, PlanDev plan);
 __global__ void k_row_offsets(const FrameDev* frames, PlanDev plan);
 __global__ void k_tile_base(const FrameDev* frames, PlanDev plan);

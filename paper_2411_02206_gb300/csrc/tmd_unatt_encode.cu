@@ -6,22 +6,31 @@
 // Per (sector,row) bin the clusters are ordered by (time, pad), ties in input
 // order, and stored as pad / time differences to the preceding cluster of the
 // bin (the first to zero), mod 2^16 / 2^32, with their charges, flags and
-// sigmas in the same order; the bins follow each other in bin order.  That is
-// one stable sort of the composite key
-//     bin << 48 | time << 16 | pad      (bin = sector * 152 + row)
-// with the input index as the value, followed by a pass that differences
-// neighbours of the same bin and gathers the charges.
+// sigmas in the same order; the bins follow each other in bin order.
 //
-// The sort is a least-significant-digit radix sort, 8 bits per pass, stable
-// by construction (every pass keeps the order of equal digits), so ties end
-// in input order.  A pass: k_rs_upsweep counts the digits of each tile of
-// kRsTile keys; k_rs_scan turns the counts into each (digit, tile)'s first
-// output position; k_rs_downsweep ranks every key within its tile (warps in
-// order, match.any among the lanes of a step) and writes it there.  A pass
-// whose digit is the same for every key (e.g. the high time bits of a frame
-// of 4000 time bins) is detected on the device and skipped: the pass kernels
-// find the current buffer and the skip flag in a small control block, so the
-// whole encoder is asynchronous.
+// The sort goes from the most significant digit down, so that a cluster moves
+// through memory once as one 16-byte record (its native record and its input
+// index) and everything else happens on chip:
+//
+//   k_ue_init     outputs that are summed into, control block
+//   k_ue_count    clusters per bin
+//   k_ue_plan     first output position of every bin; bins by size
+//   k_ue_scatter  every record to its bin's range, in any order within it
+//   k_ue_sort_warp / _block / _big
+//                 sort one bin by (time, pad, index) and write its streams: a
+//                 warp for up to kUeWarpMax clusters, a block for up to
+//                 kUeBlockMax, a large block in time slices beyond that
+//   k_ue_general  least-significant-digit radix sort of whatever the others
+//                 leave (leaves at once when there is nothing): frames with
+//                 times of 2^24 and more, which the record does not hold, and
+//                 bins that are too large or whose times crowd too much
+//
+// A bin's sort is a distribution sort: as many buckets as clusters, equally
+// wide between the bin's first and last time, so a bucket holds about one
+// cluster and a few comparisons finish it.  The previous form, eight stable
+// radix passes over 64-bit keys and a random gather of the charges, moved each
+// cluster nine times: 3.60 ms for 20 M clusters against 0.72 ms now, and 0.193 ms
+// in 35 launches for 100 k clusters against 0.058 ms in 8.
 #include <algorithm>
 #include <cstring>
 
@@ -31,17 +40,37 @@
 namespace tmd {
 namespace {
 
+constexpr uint32_t kUeWarpMax = 128;      // clusters of a bin sorted by one warp
+constexpr uint32_t kUeBlockMax = 4096;    // by one block of kUeBlockThreads
+constexpr int kUeBlockThreads = 512;
+constexpr uint32_t kUeSliceCap = 16384;   // by one block of kUeBigThreads, per time slice
+constexpr uint32_t kUeSliceMean = 12288;  // aimed at, leaving room for uneven times
+constexpr int kUeBigThreads = 1024;
+constexpr uint32_t kUeBigMax = 1u << 18;  // larger bins: the general sort (a slice re-reads
+                                          // its whole bin, so the work grows with the square)
+constexpr uint32_t kUeBucketMax = 64;     // clusters of a bucket that one thread may sort
+constexpr int kUeScatThreads = 512;
+constexpr uint32_t kUeSpin = 1u << 22;
+
 constexpr int kRsThreads = 256;
 constexpr int kRsPerThread = 8;
 constexpr uint32_t kRsTile = kRsThreads * kRsPerThread;  // keys per tile
-constexpr int kRsPasses = 8;                             // 64-bit keys, 8-bit digits
 constexpr int kRsWarps = kRsThreads / 32;
 
-// control block: cur[0..kRsPasses] (buffer holding the keys before pass p),
-// skip[0..kRsPasses) (pass p is skipped)
-struct RsCtl {
-  uint32_t cur[kRsPasses + 1];
-  uint32_t skip[kRsPasses];
+// Zeroed by k_ue_init, lists and counts written by k_ue_plan.
+struct UeCtl {
+  uint32_t wide;               // a time of 2^24 or more: everything in the general sort
+  uint32_t n_general;          // bins marked for the general sort
+  uint32_t n_block, n_big;     // bins in the lists
+  uint32_t next_block, next_big;
+  uint32_t barrier;            // arrivals at the general sort's grid barriers
+  uint32_t pad;
+  uint32_t general[kNBin];     // marks
+};
+struct UePlan {
+  uint32_t start[kNBin + 1];   // first output position of every bin
+  uint32_t cursor[kNBin];      // next free record of every bin during the scatter
+  uint32_t block[kNBin], big[kNBin];
 };
 
 struct UeArgs {
@@ -64,55 +93,55 @@ struct UeArgs {
   uint8_t* sigp_o;
   uint8_t* sigt_o;
   uint32_t* status;
+  int vec;  // every input aligned for loads of four clusters
 };
 
-// Composite keys and input indices; clusters per bin; a row >= 152 or a
-// sector >= 36 sets TMD_STATUS_ROW (the cluster is then counted in bin 5471).
-__global__ void __launch_bounds__(256) k_ue_keys(UeArgs a, uint64_t* keys, uint32_t* vals,
-                                                 RsCtl* ctl) {
+// Bin of a cluster; a row >= 152 or a sector >= 36 counts in bin 5471.
+__device__ __forceinline__ uint32_t ue_bin(uint32_t row, uint32_t sector, uint32_t& st) {
+  if (row >= (uint32_t)kNRow || sector >= (uint32_t)kNSec) {
+    st = kStRow;
+    return kNBin - 1;
+  }
+  return sector * kNRow + row;
+}
+
+__global__ void __launch_bounds__(256) k_ue_init(UeArgs a, UeCtl* ctl) {
+  const uint32_t i = blockIdx.x * 256 + threadIdx.x;
+  if (i < (uint32_t)kNBin) a.n_unatt[i] = 0u;
+  if (i < sizeof(UeCtl) / 4) reinterpret_cast<uint32_t*>(ctl)[i] = 0u;
+  if (i == 0) *a.status = 0u;
+}
+
+// Clusters per bin: counters in shared memory, added to the output once per
+// block (so a block takes at least a few thousand clusters).
+__global__ void __launch_bounds__(1024) k_ue_count(UeArgs a) {
   __shared__ uint32_t s_cnt[kNBin];
-  for (int i = threadIdx.x; i < kNBin; i += blockDim.x) s_cnt[i] = 0u;
-  if (blockIdx.x == 0 && threadIdx.x <= kRsPasses) ctl->cur[threadIdx.x] = 0u;
+  for (int i = threadIdx.x; i < kNBin; i += 1024) s_cnt[i] = 0u;
   __syncthreads();
   uint32_t st = 0;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += gridDim.x * blockDim.x) {
-    const uint32_t r = a.row[i], s = a.sector[i];
-    uint32_t b = s * kNRow + r;
-    if (r >= (uint32_t)kNRow || s >= (uint32_t)kNSec) {
-      st = kStRow;
-      b = kNBin - 1;
+  const uint32_t groups = a.n / 4 + (a.n % 4 != 0);
+  for (uint32_t g = blockIdx.x * 1024 + threadIdx.x; g < groups; g += gridDim.x * 1024) {
+    const uint32_t i = g * 4;
+    if (a.vec && a.n - i >= 4) {
+      const uint32_t r = *reinterpret_cast<const uint32_t*>(a.row + i);
+      const uint32_t s = *reinterpret_cast<const uint32_t*>(a.sector + i);
+#pragma unroll
+      for (int q = 0; q < 4; q++)
+        atomicAdd(&s_cnt[ue_bin((r >> (8 * q)) & 255u, (s >> (8 * q)) & 255u, st)], 1u);
+    } else {
+      for (uint32_t q = 0; q < 4 && q < a.n - i; q++)
+        atomicAdd(&s_cnt[ue_bin(a.row[i + q], a.sector[i + q], st)], 1u);
     }
-    keys[i] = ((uint64_t)b << 48) | ((uint64_t)a.time[i] << 16) | a.pad[i];
-    vals[i] = i;
-    atomicAdd(&s_cnt[b], 1u);
   }
   if (__syncthreads_or(st != 0) && threadIdx.x == 0) atomicOr(a.status, kStRow);
-  for (int i = threadIdx.x; i < kNBin; i += blockDim.x)
+  for (int i = threadIdx.x; i < kNBin; i += 1024)
     if (s_cnt[i]) atomicAdd(&a.n_unatt[i], s_cnt[i]);
 }
 
-// Digit counts of every tile: counts[d * n_tiles + tile].
-__global__ void __launch_bounds__(kRsThreads) k_rs_upsweep(const uint64_t* k0, const uint64_t* k1,
-                                                          uint32_t n, uint32_t shift,
-                                                          uint32_t* counts, const RsCtl* ctl,
-                                                          int pass) {
-  __shared__ uint32_t s_c[256];
-  const uint64_t* keys = ctl->cur[pass] ? k1 : k0;
-  s_c[threadIdx.x] = 0u;
-  __syncthreads();
-  const uint32_t base = blockIdx.x * kRsTile;
-#pragma unroll
-  for (int u = 0; u < kRsPerThread; u++) {
-    const uint32_t i = base + u * kRsThreads + threadIdx.x;
-    if (i < n) atomicAdd(&s_c[(uint32_t)(keys[i] >> shift) & 255u], 1u);
-  }
-  __syncthreads();
-  counts[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = s_c[threadIdx.x];
-}
-
-// Exclusive scan over a block of 256 threads; total in *tot.
-__device__ __forceinline__ uint32_t scan256(uint32_t v, uint32_t* tot) {
-  __shared__ uint32_t s_w[8];
+// Exclusive scan over a block of B threads; total in tot.
+template <int B>
+__device__ __forceinline__ uint32_t ue_scan(uint32_t v, uint32_t& tot) {
+  __shared__ uint32_t s_w[32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   uint32_t x = v;
 #pragma unroll
@@ -122,98 +151,535 @@ __device__ __forceinline__ uint32_t scan256(uint32_t v, uint32_t* tot) {
   }
   if (lane == 31) s_w[w] = x;
   __syncthreads();
-  uint32_t off = 0, all = 0;
+  // every warp scans the warp totals
+  const uint32_t t = lane < B / 32 ? s_w[lane] : 0u;
+  uint32_t y = t;
 #pragma unroll
-  for (int i = 0; i < 8; i++) {
-    off += i < w ? s_w[i] : 0u;
-    all += s_w[i];
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t z = __shfl_up_sync(0xffffffffu, y, o);
+    if (lane >= o) y += z;
   }
+  tot = __shfl_sync(0xffffffffu, y, 31);
+  const uint32_t off = __shfl_sync(0xffffffffu, y - t, w);
   __syncthreads();
-  *tot = all;
   return off + x - v;
 }
 
-// One block per digit: the tiles' exclusive offsets within the digit (in
-// place) and the digit's total.
-__global__ void __launch_bounds__(256) k_rs_scan(uint32_t* counts, uint32_t n_tiles,
-                                                 uint32_t* digit_tot) {
-  uint32_t* c = counts + (size_t)blockIdx.x * n_tiles;
-  uint32_t run = 0;
-  for (uint32_t b = 0; b < n_tiles; b += 256) {
-    const uint32_t i = b + threadIdx.x;
-    const uint32_t v = i < n_tiles ? c[i] : 0u;
-    uint32_t tot;
-    const uint32_t e = scan256(v, &tot);
-    if (i < n_tiles) c[i] = run + e;
-    run += tot;
+// One block: output positions of the bins, and which kernel sorts each.
+__global__ void __launch_bounds__(1024) k_ue_plan(UeArgs a, UePlan* plan, UeCtl* ctl) {
+  constexpr int Q = (kNBin + 1023) / 1024;
+  const uint32_t b0 = threadIdx.x * Q;
+  uint32_t v[Q], sum = 0, tot;
+#pragma unroll
+  for (int q = 0; q < Q; q++) {
+    v[q] = b0 + q < (uint32_t)kNBin ? a.n_unatt[b0 + q] : 0u;
+    sum += v[q];
   }
-  if (threadIdx.x == 0) digit_tot[blockIdx.x] = run;
+  uint32_t run = ue_scan<1024>(sum, tot);
+#pragma unroll
+  for (int q = 0; q < Q; q++) {
+    const uint32_t b = b0 + q;
+    if (b >= (uint32_t)kNBin) break;
+    plan->start[b] = plan->cursor[b] = run;
+    run += v[q];
+    if (v[q] > kUeBigMax) {
+      ctl->general[b] = 1u;
+      atomicAdd(&ctl->n_general, 1u);
+    } else if (v[q] > kUeBlockMax) {
+      plan->big[atomicAdd(&ctl->n_big, 1u)] = b;
+    } else if (v[q] > kUeWarpMax) {
+      plan->block[atomicAdd(&ctl->n_block, 1u)] = b;
+    }
+  }
+  if (threadIdx.x == 0) plan->start[kNBin] = tot;
 }
 
-// The digits' first output positions; whether the pass can be skipped (one
-// digit holds every key) and which buffer the next pass reads.
-__global__ void __launch_bounds__(256) k_rs_scan2(uint32_t* digit_tot, uint32_t n, RsCtl* ctl,
-                                                  int pass) {
-  const uint32_t v = digit_tot[threadIdx.x];
-  const bool all = v == n;
-  uint32_t tot;
-  const uint32_t e = scan256(v, &tot);
-  const bool skip = __syncthreads_or(all) != 0;
-  digit_tot[threadIdx.x] = e;
+// Records to their bins.  A block counts its clusters per bin in shared memory
+// (each cluster's count is its place among the block's clusters of the bin),
+// reserves the bins' ranges with one global atomic per bin, all in flight
+// together, and writes 16-byte records.  The order within a bin depends on the
+// blocks' timing; the sort does not, because the record carries the input index.
+// Larger tiles (G groups of four clusters per thread) reserve less often and
+// write longer runs; small frames take small tiles to occupy every SM.
+template <int G>
+__global__ void __launch_bounds__(kUeScatThreads, 2) k_ue_scatter(UeArgs a, uint4* __restrict__ rec,
+                                                                 UePlan* plan, UeCtl* ctl) {
+  constexpr int T = kUeScatThreads;
+  constexpr int Q = (kNBin + T - 1) / T;
+  __shared__ uint32_t s_cnt[kNBin];
+  const uint32_t tid = threadIdx.x;
+  for (int i = tid; i < kNBin; i += T) s_cnt[i] = 0u;
+  __syncthreads();
+  const uint32_t base = blockIdx.x * (uint32_t)(T * 4 * G);
+  const uint32_t cnt = min((uint32_t)(T * 4 * G), a.n - base);
+  uint32_t kr[4 * G];  // bin | place in the block's clusters of the bin << 13
+  uint32_t st = 0;
+#pragma unroll
+  for (int g = 0; g < G; g++) {
+    const uint32_t l = (g * T + tid) * 4;
+    uint32_t r = 0, s = 0;
+    if (a.vec && l + 4 <= cnt) {
+      r = *reinterpret_cast<const uint32_t*>(a.row + base + l);
+      s = *reinterpret_cast<const uint32_t*>(a.sector + base + l);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; q++)
+        if (l + q < cnt) {
+          r |= (uint32_t)a.row[base + l + q] << (8 * q);
+          s |= (uint32_t)a.sector[base + l + q] << (8 * q);
+        }
+    }
+    kr[4 * g] = r;  // row and sector bytes until they are counted
+    kr[4 * g + 1] = s;
+  }
+#pragma unroll
+  for (int g = 0; g < G; g++) {
+    const uint32_t l = (g * T + tid) * 4, r = kr[4 * g], s = kr[4 * g + 1];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      kr[4 * g + q] = 0xFFFFFFFFu;
+      if (l + q < cnt) {
+        const uint32_t b = ue_bin((r >> (8 * q)) & 255u, (s >> (8 * q)) & 255u, st);
+        kr[4 * g + q] = b | (atomicAdd(&s_cnt[b], 1u) << 13);
+      }
+    }
+  }
+  __syncthreads();
+  uint32_t c[Q];
+#pragma unroll
+  for (int q = 0; q < Q; q++) {
+    const uint32_t b = tid + q * T;
+    c[q] = b < (uint32_t)kNBin ? s_cnt[b] : 0u;
+    if (c[q]) c[q] = atomicAdd(&plan->cursor[b], c[q]);
+  }
+#pragma unroll
+  for (int q = 0; q < Q; q++)
+    if (tid + q * T < (uint32_t)kNBin) s_cnt[tid + q * T] = c[q];
+  __syncthreads();
+  bool wide = false;
+#pragma unroll
+  for (int g = 0; g < G; g++) {
+    const uint32_t l = (g * T + tid) * 4, i = base + l;
+    uint32_t tm[4] = {}, pd[4] = {}, qt[4] = {}, qm[4] = {}, fl = 0, sp = 0, sg = 0;
+    if (a.vec && l + 4 <= cnt) {
+      const uint4 t = *reinterpret_cast<const uint4*>(a.time + i);
+      const uint2 p = *reinterpret_cast<const uint2*>(a.pad + i);
+      const uint2 x = *reinterpret_cast<const uint2*>(a.qtot + i);
+      const uint2 y = *reinterpret_cast<const uint2*>(a.qmax + i);
+      fl = *reinterpret_cast<const uint32_t*>(a.flags + i);
+      sp = *reinterpret_cast<const uint32_t*>(a.sigp + i);
+      sg = *reinterpret_cast<const uint32_t*>(a.sigt + i);
+      tm[0] = t.x; tm[1] = t.y; tm[2] = t.z; tm[3] = t.w;
+      pd[0] = p.x & 0xFFFFu; pd[1] = p.x >> 16; pd[2] = p.y & 0xFFFFu; pd[3] = p.y >> 16;
+      qt[0] = x.x & 0xFFFFu; qt[1] = x.x >> 16; qt[2] = x.y & 0xFFFFu; qt[3] = x.y >> 16;
+      qm[0] = y.x & 0xFFFFu; qm[1] = y.x >> 16; qm[2] = y.y & 0xFFFFu; qm[3] = y.y >> 16;
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; q++)
+        if (l + q < cnt) {
+          tm[q] = a.time[i + q];
+          pd[q] = a.pad[i + q];
+          qt[q] = a.qtot[i + q];
+          qm[q] = a.qmax[i + q];
+          fl |= (uint32_t)a.flags[i + q] << (8 * q);
+          sp |= (uint32_t)a.sigp[i + q] << (8 * q);
+          sg |= (uint32_t)a.sigt[i + q] << (8 * q);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      const uint32_t k = kr[4 * g + q];
+      if (k == 0xFFFFFFFFu) continue;
+      wide |= (tm[q] >> 24) != 0;
+      rec[s_cnt[k & 8191u] + (k >> 13)] =
+          make_uint4((tm[q] & 0xFFFFFFu) | ((fl >> (8 * q)) << 24),
+                     pd[q] | (((sg >> (8 * q)) & 255u) << 16) | ((sp >> (8 * q)) << 24),
+                     qm[q] | (qt[q] << 16), i + q);
+    }
+  }
+  if (__syncthreads_or(wide) && tid == 0) ctl->wide = 1u;
+}
+
+// The encoded cluster at output position p.
+__device__ __forceinline__ void ue_emit(const UeArgs& a, uint32_t p, uint32_t pad_diff,
+                                        uint32_t time_diff, const uint4& r) {
+  a.pad_diff[p] = (uint16_t)pad_diff;
+  a.time_diff[p] = time_diff;
+  a.qtot_o[p] = (uint16_t)(r.z >> 16);
+  a.qmax_o[p] = (uint16_t)r.z;
+  a.flags_o[p] = (uint8_t)(r.x >> 24);
+  a.sigp_o[p] = (uint8_t)(r.y >> 24);
+  a.sigt_o[p] = (uint8_t)(r.y >> 16);
+}
+
+// (time, pad) of a record: 40 bits.
+__device__ __forceinline__ uint64_t ue_key(uint32_t x, uint32_t y) {
+  return ((uint64_t)(x & 0xFFFFFFu) << 16) | (y & 0xFFFFu);
+}
+
+// One warp per bin of up to kUeWarpMax clusters: every lane counts, for each
+// of its records, the records that come before it.
+__global__ void __launch_bounds__(256) k_ue_sort_warp(UeArgs a, const uint4* __restrict__ rec,
+                                                     const UePlan* plan, const UeCtl* ctl) {
+  constexpr int E = kUeWarpMax / 32;
+  __shared__ uint4 s_rec[8][kUeWarpMax];
+  __shared__ uint8_t s_ord[8][kUeWarpMax];
+  const uint32_t w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t b = blockIdx.x * 8 + w;
+  if (b >= (uint32_t)kNBin || ctl->wide) return;
+  const uint32_t s0 = plan->start[b], n = plan->start[b + 1] - s0;
+  if (n == 0 || n > kUeWarpMax) return;
+  uint4 r[E];
+  uint32_t rank[E];
+#pragma unroll
+  for (int u = 0; u < E; u++) {
+    const uint32_t e = lane + 32 * u;
+    rank[u] = 0;
+    r[u] = e < n ? rec[s0 + e] : make_uint4(0, 0, 0, 0);
+    if (e < n) s_rec[w][e] = r[u];
+  }
+  __syncwarp();
+  const uint32_t eu = (n + 31) / 32;
+  for (uint32_t j = 0; j < n; j++) {
+    const uint4 o = s_rec[w][j];
+    const uint64_t ko = ue_key(o.x, o.y);
+#pragma unroll
+    for (int u = 0; u < E; u++)
+      if ((uint32_t)u < eu) {
+        const uint64_t k = ue_key(r[u].x, r[u].y);
+        rank[u] += (ko < k || (ko == k && o.w < r[u].w)) ? 1u : 0u;
+      }
+  }
+#pragma unroll
+  for (int u = 0; u < E; u++)
+    if (lane + 32 * u < n) s_ord[w][rank[u]] = (uint8_t)(lane + 32 * u);
+  __syncwarp();
+  for (uint32_t q = lane; q < n; q += 32) {
+    const uint4 v = s_rec[w][s_ord[w][q]];
+    const uint4 o = q ? s_rec[w][s_ord[w][q - 1]] : make_uint4(0, 0, 0, 0);
+    ue_emit(a, s0 + q, v.y - o.y, (v.x & 0xFFFFFFu) - (o.x & 0xFFFFFFu), v);
+  }
+}
+
+// Buckets of a bin (or time slice): d is the distance of a cluster's leading
+// 32 key bits (time, high byte of the pad) from the first one's, below width.
+struct UeBuckets {
+  uint32_t mul;  // 0: one bucket per value
+  __device__ __forceinline__ void init(uint64_t width, uint32_t n_buckets) {
+    // at most n_buckets / width * 2^32: the factor covers the three roundings
+    mul = width <= n_buckets
+              ? 0u
+              : (uint32_t)(__fdividef((float)n_buckets * 4294967296.0f, (float)width) * 0.99999f);
+  }
+  __device__ __forceinline__ uint32_t of(uint32_t d) const { return mul ? __umulhi(d, mul) : d; }
+};
+
+// Insertion sort of one bucket's entries ((time, pad) << 24 | place in the
+// bin); equal (time, pad) by input index.
+__device__ __forceinline__ void ue_sort_bucket(uint64_t* k, uint32_t lo, uint32_t hi,
+                                               const uint4* rec) {
+  for (uint32_t i = lo + 1; i < hi; i++) {
+    const uint64_t x = k[i];
+    uint32_t j = i;
+    while (j > lo) {
+      const uint64_t y = k[j - 1];
+      bool after = y > x;
+      if ((y >> 24) == (x >> 24))
+        after = rec[(uint32_t)y & 0xFFFFFFu].w > rec[(uint32_t)x & 0xFFFFFFu].w;
+      if (!after) break;
+      k[j] = y;
+      j--;
+    }
+    k[j] = x;
+  }
+}
+
+// Streams of n sorted entries from output position p0; prev is the entry
+// before the first (0: none, differences to zero).
+template <int B>
+__device__ __forceinline__ void ue_emit_sorted(const UeArgs& a, uint32_t p0, uint32_t n,
+                                               const uint64_t* k, uint64_t prev,
+                                               const uint4* __restrict__ rec) {
+#pragma unroll 2
+  for (uint32_t q = threadIdx.x; q < n; q += B) {
+    const uint64_t x = k[q], y = q ? k[q - 1] : prev;
+    const uint4 r = rec[(uint32_t)x & 0xFFFFFFu];
+    ue_emit(a, p0 + q, (uint32_t)(x >> 24) - (uint32_t)(y >> 24),
+            (uint32_t)(x >> 40) - (uint32_t)(y >> 40), r);
+  }
+}
+
+__device__ __forceinline__ void ue_mark_general(UeCtl* ctl, uint32_t b) {
+  if (atomicExch(&ctl->general[b], 1u) == 0u) atomicAdd(&ctl->n_general, 1u);
+}
+
+// Smallest and largest value over the block, through s (2 x 32 words).
+__device__ __forceinline__ void ue_minmax(uint32_t& lo, uint32_t& hi, uint32_t* s, int warps) {
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  const uint32_t lane = threadIdx.x & 31;
+  if (lane == 0) {
+    s[threadIdx.x >> 5] = lo;
+    s[32 + (threadIdx.x >> 5)] = hi;
+  }
+  __syncthreads();
+  lo = __reduce_min_sync(0xffffffffu, lane < (uint32_t)warps ? s[lane] : 0xFFFFFFFFu);
+  hi = __reduce_max_sync(0xffffffffu, lane < (uint32_t)warps ? s[32 + lane] : 0u);
+}
+
+// Blocks take the listed bins in turn.  A thread keeps its eight clusters'
+// keys in registers; their records are read again, from the caches, when the
+// sorted streams are written.
+__global__ void __launch_bounds__(kUeBlockThreads, 3) k_ue_sort_block(UeArgs a, const uint4* rec,
+                                                                     const UePlan* plan,
+                                                                     UeCtl* ctl) {
+  constexpr int T = kUeBlockThreads, E = kUeBlockMax / T;
+  extern __shared__ uint64_t s_dyn[];
+  uint64_t* s_key = s_dyn;                                            // kUeBlockMax
+  uint32_t* s_cnt = reinterpret_cast<uint32_t*>(s_dyn + kUeBlockMax);  // kUeBlockMax
+  __shared__ uint32_t s_task, s_mm[64];
+  const uint32_t tid = threadIdx.x;
+  const uint32_t n_list = ctl->wide ? 0u : ctl->n_block;
+  for (;;) {
+    if (tid == 0) s_task = atomicAdd(&ctl->next_block, 1u);
+    __syncthreads();
+    const uint32_t task = s_task;
+    if (task >= n_list) break;
+    const uint32_t b = plan->block[task];
+    const uint32_t s0 = plan->start[b], n = plan->start[b + 1] - s0;
+    const uint4* __restrict__ r0 = rec + s0;
+    uint2 w[E];
+    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+#pragma unroll
+    for (int u = 0; u < E; u++) {
+      const uint32_t e = tid + u * T;
+      if (e < n) w[u] = *reinterpret_cast<const uint2*>(r0 + e);
+    }
+#pragma unroll
+    for (int u = 0; u < E; u++) s_cnt[tid + u * T] = 0u;
+#pragma unroll
+    for (int u = 0; u < E; u++)
+      if (tid + u * T < n) {
+        const uint32_t d = (w[u].x << 8) | ((w[u].y >> 8) & 255u);
+        lo = min(lo, d);
+        hi = max(hi, d);
+      }
+    ue_minmax(lo, hi, s_mm, T / 32);
+    UeBuckets bk;
+    bk.init((uint64_t)(hi - lo) + 1, n);
+    uint32_t br[E];
+#pragma unroll
+    for (int u = 0; u < E; u++)
+      if (tid + u * T < n) {
+        const uint32_t d = (w[u].x << 8) | ((w[u].y >> 8) & 255u);
+        const uint32_t k = bk.of(d - lo);
+        br[u] = k | (atomicAdd(&s_cnt[k], 1u) << 16);
+      }
+    __syncthreads();
+    // first entry of every bucket, E consecutive buckets per thread
+    uint32_t c[E], sum = 0, most = 0, tot;
+#pragma unroll
+    for (int u = 0; u < E; u++) {
+      c[u] = s_cnt[tid * E + u];
+      sum += c[u];
+      most = max(most, c[u]);
+    }
+    uint32_t run = ue_scan<T>(sum, tot);
+#pragma unroll
+    for (int u = 0; u < E; u++) {
+      s_cnt[tid * E + u] = run;
+      run += c[u];
+    }
+    if (__syncthreads_or(most > kUeBucketMax)) {
+      if (tid == 0) ue_mark_general(ctl, b);
+      continue;
+    }
+#pragma unroll
+    for (int u = 0; u < E; u++)
+      if (tid + u * T < n)
+        s_key[s_cnt[br[u] & 0xFFFFu] + (br[u] >> 16)] =
+            (ue_key(w[u].x, w[u].y) << 24) | (tid + u * T);
+    __syncthreads();
+    for (uint32_t k = tid; k < n; k += T) {
+      const uint32_t k0 = s_cnt[k], k1 = k + 1 < n ? s_cnt[k + 1] : n;
+      if (k1 > k0 + 1) ue_sort_bucket(s_key, k0, k1, r0);
+    }
+    __syncthreads();
+    ue_emit_sorted<T>(a, s0, n, s_key, 0ull, r0);
+  }
+}
+
+// Larger bins, one large block each: the bin is cut into equal time slices
+// of about kUeSliceMean clusters, sorted and written one after the other.
+__global__ void __launch_bounds__(kUeBigThreads, 1) k_ue_sort_big(UeArgs a, const uint4* rec,
+                                                                 const UePlan* plan, UeCtl* ctl) {
+  constexpr int T = kUeBigThreads, E = kUeSliceCap / T;
+  extern __shared__ uint64_t s_dyn[];
+  uint64_t* s_key = s_dyn;                                            // kUeSliceCap
+  uint32_t* s_cnt = reinterpret_cast<uint32_t*>(s_dyn + kUeSliceCap);  // kUeSliceCap
+  __shared__ uint32_t s_task, s_mm[64];
+  const uint32_t tid = threadIdx.x;
+  const uint32_t n_list = ctl->wide ? 0u : ctl->n_big;
+  for (;;) {
+    if (tid == 0) s_task = atomicAdd(&ctl->next_big, 1u);
+    __syncthreads();
+    const uint32_t task = s_task;
+    if (task >= n_list) break;
+    const uint32_t b = plan->big[task];
+    const uint32_t s0 = plan->start[b], n = plan->start[b + 1] - s0;
+    const uint4* __restrict__ r0 = rec + s0;
+    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+#pragma unroll 4
+    for (uint32_t e = tid; e < n; e += T) {
+      const uint2 w = *reinterpret_cast<const uint2*>(r0 + e);
+      const uint32_t d = (w.x << 8) | ((w.y >> 8) & 255u);
+      lo = min(lo, d);
+      hi = max(hi, d);
+    }
+    ue_minmax(lo, hi, s_mm, T / 32);
+    const uint32_t slices = (n + kUeSliceMean - 1) / kUeSliceMean;
+    const uint64_t width = (uint64_t)(hi - lo) / slices + 1;
+    UeBuckets bk;
+    bk.init(width, kUeSliceCap);
+    uint32_t out = 0;
+    uint64_t prev = 0ull;
+    for (uint32_t s = 0; s < slices && out < n; s++) {
+      const uint64_t d0 = (uint64_t)lo + s * width;
+#pragma unroll
+      for (int u = 0; u < E; u++) s_cnt[tid + u * T] = 0u;
+      __syncthreads();
+#pragma unroll 4
+      for (uint32_t e = tid; e < n; e += T) {
+        const uint2 w = *reinterpret_cast<const uint2*>(r0 + e);
+        const uint32_t d = (w.x << 8) | ((w.y >> 8) & 255u);
+        if (d >= d0 && d - d0 < width) atomicAdd(&s_cnt[bk.of((uint32_t)(d - d0))], 1u);
+      }
+      __syncthreads();
+      uint32_t c[E], sum = 0, most = 0, m;
+#pragma unroll
+      for (int u = 0; u < E; u++) {
+        c[u] = s_cnt[tid * E + u];
+        sum += c[u];
+        most = max(most, c[u]);
+      }
+      uint32_t run = ue_scan<T>(sum, m);
+#pragma unroll
+      for (int u = 0; u < E; u++) {
+        s_cnt[tid * E + u] = run;
+        run += c[u];
+      }
+      if (__syncthreads_or(most > kUeBucketMax) || m > kUeSliceCap) {
+        if (tid == 0) ue_mark_general(ctl, b);
+        break;  // the general sort writes the whole bin
+      }
+#pragma unroll 4
+      for (uint32_t e = tid; e < n; e += T) {
+        const uint2 w = *reinterpret_cast<const uint2*>(r0 + e);
+        const uint32_t d = (w.x << 8) | ((w.y >> 8) & 255u);
+        if (d >= d0 && d - d0 < width)
+          s_key[atomicAdd(&s_cnt[bk.of((uint32_t)(d - d0))], 1u)] = (ue_key(w.x, w.y) << 24) | e;
+      }
+      __syncthreads();  // s_cnt[k] is now the end of bucket k
+#pragma unroll 1
+      for (uint32_t k = tid; k < kUeSliceCap; k += T) {
+        const uint32_t k0 = k ? s_cnt[k - 1] : 0u, k1 = s_cnt[k];
+        if (k1 > k0 + 1) ue_sort_bucket(s_key, k0, k1, r0);
+      }
+      __syncthreads();
+      ue_emit_sorted<T>(a, s0 + out, m, s_key, prev, r0);
+      if (m) prev = s_key[m - 1];
+      out += m;
+      __syncthreads();
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// General sort: 8-bit radix passes, least significant first, by one
+// cooperative launch.  Entry: {time, index, bin << 16 | pad, 0}.
+// ---------------------------------------------------------------------------
+
+// All blocks of the (cooperative) launch; false if they did not all arrive
+// within kUeSpin polls.
+__device__ __forceinline__ bool ue_grid_barrier(uint32_t* arrivals, uint32_t& target) {
+  __shared__ int s_ok;
+  target += gridDim.x;
+  __syncthreads();
   if (threadIdx.x == 0) {
-    ctl->skip[pass] = skip ? 1u : 0u;
-    ctl->cur[pass + 1] = skip ? ctl->cur[pass] : ctl->cur[pass] ^ 1u;
+    __threadfence();
+    atomicAdd(arrivals, 1u);
+    int ok = 0;
+    for (uint32_t i = 0; i < kUeSpin && !ok; i++) {
+      ok = (int32_t)(*(volatile uint32_t*)arrivals - target) >= 0;
+      if (!ok) __nanosleep(64);
+    }
+    __threadfence();
+    s_ok = ok;
   }
+  __syncthreads();
+  return s_ok != 0;
 }
 
-// Stable scatter of one pass.  Warp w of a tile takes keys [w * 256, w * 256 +
-// 256) of the tile in steps of 32; a key's place is its digit's first
-// position, plus the tile's offset within the digit, plus the keys of that
-// digit in the tile's earlier warps and earlier steps and lanes.
-__global__ void __launch_bounds__(kRsThreads) k_rs_downsweep(uint64_t* k0, uint32_t* v0,
-                                                            uint64_t* k1, uint32_t* v1,
-                                                            uint32_t n, uint32_t shift,
-                                                            const uint32_t* counts,
-                                                            const uint32_t* digit_base,
-                                                            const RsCtl* ctl, int pass) {
-  __shared__ uint32_t s_wc[kRsWarps][256];
-  if (ctl->skip[pass]) return;  // the same for every block
-  const bool from1 = ctl->cur[pass] != 0u;
-  const uint64_t* __restrict__ sk = from1 ? k1 : k0;
-  const uint32_t* __restrict__ sv = from1 ? v1 : v0;
-  uint64_t* __restrict__ dk = from1 ? k0 : k1;
-  uint32_t* __restrict__ dv = from1 ? v0 : v1;
+__device__ __forceinline__ uint32_t rs_digit(const uint4& e, int pass) {
+  const uint32_t w = pass < 4 ? e.y : (pass < 6 ? e.z & 0xFFFFu : (pass < 10 ? e.x : e.z >> 16));
+  const int sh = pass < 4 ? pass : (pass < 6 ? pass - 4 : (pass < 10 ? pass - 6 : pass - 10));
+  return (w >> (8 * sh)) & 255u;
+}
+
+__device__ __forceinline__ void rs_upsweep(const uint4* src, uint32_t m, uint32_t tile,
+                                           uint32_t n_tiles, int pass, uint32_t* counts,
+                                           uint32_t* s_c) {
+  s_c[threadIdx.x] = 0u;
+  __syncthreads();
+  const uint32_t base = tile * kRsTile;
+#pragma unroll
+  for (int u = 0; u < kRsPerThread; u++) {
+    const uint32_t l = u * kRsThreads + threadIdx.x;
+    if (l < m - base) atomicAdd(&s_c[rs_digit(__ldcg(src + base + l), pass)], 1u);
+  }
+  __syncthreads();
+  counts[(size_t)threadIdx.x * n_tiles + tile] = s_c[threadIdx.x];
+  __syncthreads();
+}
+
+// Stable scatter of one tile.  Warp w takes entries [w * 256, w * 256 + 256)
+// of the tile in steps of 32; an entry's place is its digit's first position,
+// plus the tile's offset within the digit, plus the entries of that digit in
+// the tile's earlier warps and earlier steps and lanes.
+__device__ __forceinline__ void rs_downsweep(const uint4* src, uint4* dst, uint32_t m,
+                                             uint32_t tile, uint32_t n_tiles, int pass,
+                                             const uint32_t* counts, const uint32_t* s_base,
+                                             uint32_t (*s_wc)[256]) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int i = threadIdx.x; i < kRsWarps * 256; i += kRsThreads) (&s_wc[0][0])[i] = 0u;
   __syncthreads();
-  const uint32_t base = blockIdx.x * kRsTile + w * (32u * kRsPerThread);
-  uint64_t key[kRsPerThread];
-  uint32_t val[kRsPerThread], dig[kRsPerThread], rk[kRsPerThread];
+  const uint32_t base = tile * kRsTile, left = m - base;
+  uint4 ent[kRsPerThread];
+  uint32_t rk[kRsPerThread];
 #pragma unroll
   for (int u = 0; u < kRsPerThread; u++) {
-    const uint32_t i = base + 32u * u + lane;
-    key[u] = i < n ? sk[i] : 0ull;
-    val[u] = i < n ? sv[i] : 0u;
+    const uint32_t l = w * (32u * kRsPerThread) + 32u * u + lane;
+    ent[u] = l < left ? __ldcg(src + base + l) : make_uint4(0, 0, 0, 0);
   }
 #pragma unroll
   for (int u = 0; u < kRsPerThread; u++) {
-    const uint32_t i = base + 32u * u + lane;
-    const bool in = i < n;
+    const uint32_t l = w * (32u * kRsPerThread) + 32u * u + lane;
+    const bool in = l < left;
     const uint32_t act = __ballot_sync(0xffffffffu, in);
-    dig[u] = (uint32_t)(key[u] >> shift) & 255u;
     rk[u] = 0;
     if (in) {
-      const uint32_t peers = __match_any_sync(act, dig[u]);
-      rk[u] = s_wc[w][dig[u]] + __popc(peers & lanemask_lt());
+      const uint32_t d = rs_digit(ent[u], pass);
+      const uint32_t peers = __match_any_sync(act, d);
+      rk[u] = s_wc[w][d] + __popc(peers & lanemask_lt());
       __syncwarp(act);
-      if (lane == __ffs(peers) - 1) s_wc[w][dig[u]] += __popc(peers);
+      if (lane == __ffs(peers) - 1) s_wc[w][d] += __popc(peers);
     }
     __syncwarp();
   }
   __syncthreads();
-  {  // per digit: the keys of the tile's earlier warps
+  {  // per digit: its first position, the tile's offset, the tile's earlier warps
     const uint32_t d = threadIdx.x;
-    uint32_t run = 0;
+    uint32_t run = s_base[d] + __ldcg(counts + (size_t)d * n_tiles + tile);
 #pragma unroll
     for (int ww = 0; ww < kRsWarps; ww++) {
       const uint32_t c = s_wc[ww][d];
@@ -222,39 +688,105 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_downsweep(uint64_t* k0, uint3
     }
   }
   __syncthreads();
-  const uint32_t n_tiles = gridDim.x;
 #pragma unroll
   for (int u = 0; u < kRsPerThread; u++) {
-    const uint32_t i = base + 32u * u + lane;
-    if (i < n) {
-      const uint32_t d = dig[u];
-      const uint32_t pos = digit_base[d] + counts[(size_t)d * n_tiles + blockIdx.x] + s_wc[w][d] +
-                           rk[u];
-      dk[pos] = key[u];
-      dv[pos] = val[u];
-    }
+    const uint32_t l = w * (32u * kRsPerThread) + 32u * u + lane;
+    if (l < left) dst[s_wc[w][rs_digit(ent[u], pass)] + rk[u]] = ent[u];
   }
+  __syncthreads();
 }
 
-// The encoded streams from the sorted keys: differences to the preceding
-// cluster of the same bin (the first of a bin to zero), charges gathered by
-// input index.
-__global__ void __launch_bounds__(256) k_ue_emit(UeArgs a, const uint64_t* k0, const uint32_t* v0,
-                                                 const uint64_t* k1, const uint32_t* v1,
-                                                 const RsCtl* ctl) {
-  const bool in1 = ctl->cur[kRsPasses] != 0u;
-  const uint64_t* __restrict__ keys = in1 ? k1 : k0;
-  const uint32_t* __restrict__ vals = in1 ? v1 : v0;
-  for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < a.n; p += gridDim.x * blockDim.x) {
-    const uint64_t k = keys[p];
-    const uint64_t q = p ? keys[p - 1] : 0ull;
-    const bool same = p && (q >> 48) == (k >> 48);
-    const uint32_t pad = (uint32_t)k & 0xFFFFu, time = (uint32_t)(k >> 16);
-    const uint32_t ppad = same ? (uint32_t)q & 0xFFFFu : 0u;
-    const uint32_t ptime = same ? (uint32_t)(q >> 16) : 0u;
-    a.pad_diff[p] = (uint16_t)((pad - ppad) & 0xFFFFu);
-    a.time_diff[p] = time - ptime;
-    const uint32_t i = vals[p];
+__global__ void __launch_bounds__(kRsThreads) k_ue_general(UeArgs a, uint4* r0, uint4* r1,
+                                                          const UePlan* plan, UeCtl* ctl,
+                                                          uint32_t* counts, uint32_t* digit_tot) {
+  const bool wide = ctl->wide != 0u;
+  if (!wide && ctl->n_general == 0u) return;  // the same for every block
+  __shared__ uint32_t s_first[kNBin + 1];     // a marked bin's first entry
+  __shared__ uint32_t s_wc[kRsWarps][256];
+  __shared__ uint32_t s_base[256];
+  const uint32_t tid = threadIdx.x;
+  const uint32_t gid = blockIdx.x * kRsThreads + tid, gn = gridDim.x * kRsThreads;
+  uint32_t target = 0, m = a.n;
+  bool ok = true;
+  if (wide) {
+    for (uint64_t i = gid; i < m; i += gn) {
+      uint32_t st = 0;
+      r1[i] = make_uint4(a.time[i], (uint32_t)i,
+                         (ue_bin(a.row[i], a.sector[i], st) << 16) | a.pad[i], 0u);
+    }
+  } else {
+    uint32_t run = 0;
+    for (uint32_t b0 = 0; b0 < (uint32_t)kNBin; b0 += kRsThreads) {
+      const uint32_t b = b0 + tid;
+      const uint32_t v = b < (uint32_t)kNBin && ctl->general[b] ? plan->start[b + 1] - plan->start[b]
+                                                                : 0u;
+      uint32_t tot;
+      const uint32_t e = ue_scan<kRsThreads>(v, tot);
+      if (b < (uint32_t)kNBin) s_first[b] = run + e;
+      run += tot;
+    }
+    m = run;
+    if (tid == 0) s_first[kNBin] = m;
+    __syncthreads();
+    for (uint64_t i = gid; i < m; i += gn) {
+      uint32_t lo = 0, hi = kNBin - 1;  // last bin whose entries start at or before i
+      while (lo < hi) {
+        const uint32_t mid = (lo + hi + 1) >> 1;
+        if (s_first[mid] <= i) lo = mid; else hi = mid - 1;
+      }
+      const uint4 r = r0[plan->start[lo] + ((uint32_t)i - s_first[lo])];
+      r1[i] = make_uint4(r.x & 0xFFFFFFu, r.w, (lo << 16) | (r.y & 0xFFFFu), 0u);
+    }
+  }
+  ok = ue_grid_barrier(&ctl->barrier, target);
+  const uint32_t n_tiles = m / kRsTile + (m % kRsTile != 0);
+  uint4* src = r1;
+  uint4* dst = r0;
+  // index bytes (in a wide frame the entries are in input order already),
+  // pad, time, bin; a digit that all entries share needs no pass
+  for (int pass = wide ? 4 : 0; pass < 12 && ok; pass++) {
+    for (uint32_t t = blockIdx.x; t < n_tiles; t += gridDim.x)
+      rs_upsweep(src, m, t, n_tiles, pass, counts, s_base);
+    if (!(ok = ue_grid_barrier(&ctl->barrier, target))) break;
+    for (uint32_t d = blockIdx.x; d < 256; d += gridDim.x) {
+      uint32_t* c = counts + (size_t)d * n_tiles;
+      uint32_t run = 0;
+      for (uint64_t t0 = 0; t0 < n_tiles; t0 += kRsThreads) {
+        const uint32_t v = t0 + tid < n_tiles ? __ldcg(c + t0 + tid) : 0u;
+        uint32_t tot;
+        const uint32_t e = ue_scan<kRsThreads>(v, tot);
+        if (t0 + tid < n_tiles) c[t0 + tid] = run + e;
+        run += tot;
+      }
+      if (tid == 0) digit_tot[d] = run;
+    }
+    if (!(ok = ue_grid_barrier(&ctl->barrier, target))) break;
+    const uint32_t v = __ldcg(digit_tot + tid);
+    uint32_t tot;
+    const uint32_t e = ue_scan<kRsThreads>(v, tot);
+    s_base[tid] = e;
+    if (!__syncthreads_or(v == m)) {
+      for (uint32_t t = blockIdx.x; t < n_tiles; t += gridDim.x)
+        rs_downsweep(src, dst, m, t, n_tiles, pass, counts, s_base, s_wc);
+      uint4* x = src;
+      src = dst;
+      dst = x;
+    }
+    ok = ue_grid_barrier(&ctl->barrier, target);
+  }
+  if (!ok) {
+    if (tid == 0) atomicOr(a.status, kStTimeout);
+    return;
+  }
+  for (uint64_t q = gid; q < m; q += gn) {
+    const uint4 x = __ldcg(src + q);
+    const uint4 y = q ? __ldcg(src + q - 1) : make_uint4(0, 0, 0xFFFFFFFFu, 0);
+    const uint32_t b = x.z >> 16;
+    const bool same = q && (y.z >> 16) == b;
+    const uint32_t p = wide ? (uint32_t)q : plan->start[b] + ((uint32_t)q - s_first[b]);
+    const uint32_t i = x.y;
+    a.pad_diff[p] = (uint16_t)(x.z - (same ? y.z : 0u));
+    a.time_diff[p] = x.x - (same ? y.x : 0u);
     a.qtot_o[p] = a.qtot[i];
     a.qmax_o[p] = a.qmax[i];
     a.flags_o[p] = a.flags[i];
@@ -263,7 +795,22 @@ __global__ void __launch_bounds__(256) k_ue_emit(UeArgs a, const uint64_t* k0, c
   }
 }
 
+constexpr size_t kUeBlockSmem = (size_t)kUeBlockMax * 12;
+constexpr size_t kUeBigSmem = (size_t)kUeSliceCap * 12;
+
 }  // namespace
+
+cudaError_t prepare_unatt_encode(int* blocks_per_sm) {
+  cudaError_t e = cudaFuncSetAttribute(k_ue_sort_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kUeBlockSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_ue_sort_big, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kUeBigSmem);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_ue_general, kRsThreads, 0);
+  return e;
+}
+
 }  // namespace tmd
 
 using namespace tmd;
@@ -289,23 +836,21 @@ extern "C" int tmd_encode_unattached(tmd_handle* h, const tmd_unatt_truth_in* in
   int rc = tmd_cuda_check(h, cudaSetDevice(h->device), "cudaSetDevice");
   if (rc != TMD_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const uint32_t n_tiles = n ? (n + kRsTile - 1) / kRsTile : 1u;
+  const uint32_t n_tiles = n / kRsTile + 1;
   auto up = [](size_t x) { return (x + 255) / 256 * 256; };
-  const size_t o_k0 = 0, o_k1 = up((size_t)n * 8 + 8), o_v0 = o_k1 + up((size_t)n * 8 + 8),
-               o_v1 = o_v0 + up((size_t)n * 4 + 4), o_cnt = o_v1 + up((size_t)n * 4 + 4),
-               o_dig = o_cnt + up((size_t)256 * n_tiles * 4), o_ctl = o_dig + up(256 * 4),
-               total = o_ctl + up(sizeof(RsCtl));
+  const size_t o_r0 = 0, o_r1 = up((size_t)n * 16 + 16), o_cnt = o_r1 + up((size_t)n * 16 + 16),
+               o_dig = o_cnt + up((size_t)256 * n_tiles * 4), o_plan = o_dig + up(256 * 4),
+               o_ctl = o_plan + up(sizeof(UePlan)), total = o_ctl + up(sizeof(UeCtl));
   if ((rc = h->ensure_scratch(total)) != TMD_OK) return rc;
   bool order = false;
   if ((rc = h->order_after_previous(st, &order)) != TMD_OK) return rc;
   char* base = static_cast<char*>(h->scratch);
-  uint64_t* k0 = reinterpret_cast<uint64_t*>(base + o_k0);
-  uint64_t* k1 = reinterpret_cast<uint64_t*>(base + o_k1);
-  uint32_t* v0 = reinterpret_cast<uint32_t*>(base + o_v0);
-  uint32_t* v1 = reinterpret_cast<uint32_t*>(base + o_v1);
+  uint4* r0 = reinterpret_cast<uint4*>(base + o_r0);
+  uint4* r1 = reinterpret_cast<uint4*>(base + o_r1);
   uint32_t* cnt = reinterpret_cast<uint32_t*>(base + o_cnt);
   uint32_t* dig = reinterpret_cast<uint32_t*>(base + o_dig);
-  RsCtl* ctl = reinterpret_cast<RsCtl*>(base + o_ctl);
+  UePlan* plan = reinterpret_cast<UePlan*>(base + o_plan);
+  UeCtl* ctl = reinterpret_cast<UeCtl*>(base + o_ctl);
   UeArgs a;
   a.n = n;
   a.row = in->row; a.sector = in->sector; a.pad = in->pad; a.time = in->time;
@@ -314,21 +859,34 @@ extern "C" int tmd_encode_unattached(tmd_handle* h, const tmd_unatt_truth_in* in
   a.n_unatt = out->n_unatt; a.pad_diff = out->pad_diff_u; a.time_diff = out->time_diff_u;
   a.qtot_o = out->qtot_u; a.qmax_o = out->qmax_u; a.flags_o = out->flags_u;
   a.sigp_o = out->sigma_pad_u; a.sigt_o = out->sigma_time_u; a.status = out->status;
-  rc = tmd_cuda_check(h, cudaMemsetAsync(out->n_unatt, 0, (size_t)kNBin * 4, st), "memset");
-  if (rc == TMD_OK) rc = tmd_cuda_check(h, cudaMemsetAsync(out->status, 0, 4, st), "memset");
-  if (rc != TMD_OK) return rc;
-  const uint32_t grid = std::min<uint32_t>(std::max<uint32_t>(1u, (n + 255) / 256),
-                                           (uint32_t)h->sms * 4);
-  k_ue_keys<<<grid, 256, 0, st>>>(a, k0, v0, ctl);
+  a.vec = !(mis(a.row, 4) || mis(a.sector, 4) || mis(a.flags, 4) || mis(a.sigp, 4) ||
+            mis(a.sigt, 4) || mis(a.pad, 8) || mis(a.qtot, 8) || mis(a.qmax, 8) || mis(a.time, 16));
+  const uint32_t sms = (uint32_t)h->sms;
+  k_ue_init<<<(kNBin + 9 + 255) / 256, 256, 0, st>>>(a, ctl);
   if (n) {
-    for (int p = 0; p < kRsPasses; p++) {
-      const uint32_t shift = 8u * p;
-      k_rs_upsweep<<<n_tiles, kRsThreads, 0, st>>>(k0, k1, n, shift, cnt, ctl, p);
-      k_rs_scan<<<256, 256, 0, st>>>(cnt, n_tiles, dig);
-      k_rs_scan2<<<1, 256, 0, st>>>(dig, n, ctl, p);
-      k_rs_downsweep<<<n_tiles, kRsThreads, 0, st>>>(k0, v0, k1, v1, n, shift, cnt, dig, ctl, p);
-    }
-    k_ue_emit<<<grid, 256, 0, st>>>(a, k0, v0, k1, v1, ctl);
+    k_ue_count<<<std::min(2 * sms, n / 8192 + 1), 1024, 0, st>>>(a);
+    k_ue_plan<<<1, 1024, 0, st>>>(a, plan, ctl);
+    // the largest tile that still gives every SM two blocks
+    auto tiles = [n](uint32_t g) { return n / (kUeScatThreads * 4 * g) + (n % (kUeScatThreads * 4 * g) != 0); };
+    if (tiles(8) >= 2 * sms)
+      k_ue_scatter<8><<<tiles(8), kUeScatThreads, 0, st>>>(a, r0, plan, ctl);
+    else if (tiles(2) >= 2 * sms)
+      k_ue_scatter<2><<<tiles(2), kUeScatThreads, 0, st>>>(a, r0, plan, ctl);
+    else
+      k_ue_scatter<1><<<tiles(1), kUeScatThreads, 0, st>>>(a, r0, plan, ctl);
+    k_ue_sort_warp<<<(kNBin + 7) / 8, 256, 0, st>>>(a, r0, plan, ctl);
+    if (n > kUeWarpMax)
+      k_ue_sort_block<<<std::min(3 * sms, n / kUeWarpMax), kUeBlockThreads, kUeBlockSmem, st>>>(
+          a, r0, plan, ctl);
+    if (n > kUeBlockMax)
+      k_ue_sort_big<<<std::min(sms, n / kUeBlockMax), kUeBigThreads, kUeBigSmem, st>>>(a, r0, plan,
+                                                                                    ctl);
+    void* args[] = {&a, &r0, &r1, &plan, &ctl, &cnt, &dig};
+    const uint32_t grid = std::min(n_tiles, sms * (uint32_t)h->occ_ue);
+    rc = tmd_cuda_check(h, cudaLaunchCooperativeKernel((const void*)k_ue_general, dim3(grid),
+                                                       dim3(kRsThreads), args, 0, st),
+                        "general sort launch");
+    if (rc != TMD_OK) return rc;
   }
   rc = tmd_cuda_check(h, cudaGetLastError(), "unattached encoder launch");
   if (rc != TMD_OK) return rc;
