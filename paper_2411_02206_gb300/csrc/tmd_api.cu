@@ -248,8 +248,7 @@ extern "C" int tmd_create(const tmd_config* cfg, tmd_handle** out) {
       (rc = tmd_cuda_check(h, occupancy_track_decode(0, &h->occ_decode_v[0]), "occupancy")) != TMD_OK ||
       (rc = tmd_cuda_check(h, occupancy_track_decode(1, &h->occ_decode_v[1]), "occupancy")) != TMD_OK ||
       (rc = tmd_cuda_check(h, occupancy_unatt_decode(&h->occ_unatt), "occupancy")) != TMD_OK ||
-      (rc = tmd_cuda_check(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                                  &h->occ_encode, k_track_encode, 256, 0), "occupancy")) != TMD_OK) {
+      (rc = tmd_cuda_check(h, prepare_track_encode(&h->occ_encode), "occupancy")) != TMD_OK) {
     delete h;
     return rc;
   }
@@ -542,8 +541,10 @@ int tmd_enqueue(tmd_handle* h, uint32_t nf, const tmd_frame_in* in, const tmd_fr
                                                             trace->state);
   } else if (encode) {
     if (n_warp) {
-      const uint32_t grid = std::min<uint32_t>(n_warp / 8 + 1, (uint32_t)(h->sms * h->occ_encode));
-      timed(kKTrackEncode, [&] { k_track_encode<<<grid, 256, 0, st>>>(denc, dframes, P, n_warp); });
+      const uint32_t per_block = kDecodeThreads / 32;
+      const uint32_t grid = std::min<uint32_t>((n_warp + per_block - 1) / per_block,
+                                               (uint32_t)(h->sms * h->occ_encode));
+      timed(kKTrackEncode, [&] { launch_track_encode(grid, st, denc, dframes, P, n_warp); });
     }
   } else {
     // track decode (keys, pad and time codes), per-tile counts and ranks, row

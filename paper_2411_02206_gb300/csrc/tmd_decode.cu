@@ -325,12 +325,70 @@ __global__ void k_track_trace(const FrameDev* frames, const uint32_t* ids, uint3
   }
 }
 
-__global__ void __launch_bounds__(256) k_track_encode(const EncDev* enc, const FrameDev* frames,
-                                                      PlanDev plan, uint32_t n_tasks) {
+// ---------------------------------------------------------------------------
+// Encoder staging: 14 copies of 16-byte aligned windows per lane and round of
+// 16 clusters (row, sector and leg 2 each, pad 3, time 5).  A round advances every stream by a multiple
+// of 16 bytes, so the offset of a round's first cluster in its windows is a
+// constant of the track.
+// ---------------------------------------------------------------------------
+namespace {
+
+constexpr int kEncRound = 16;
+
+// Copies the 16-byte windows from the one that holds `first` up to byte `end`
+// (at most W of them).
+template <int W>
+__device__ __forceinline__ void cp_windows(const uint32_t* dst_smem, const void* first,
+                                           const void* end) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst_smem);
+  const uintptr_t w = reinterpret_cast<uintptr_t>(first) & ~(uintptr_t)15;
+  const uintptr_t e = reinterpret_cast<uintptr_t>(end);
+#pragma unroll
+  for (int c = 0; c < W; c++)
+    if (w + 16 * c < e)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d + 16 * c), "l"(w + 16 * c)
+                   : "memory");
+}
+
+// Offset of a byte in its window.
+__device__ __forceinline__ int win_off(const void* p) {
+  return (int)(reinterpret_cast<uintptr_t>(p) & 15);
+}
+
+struct EncStage {
+  static constexpr int kSec = 8, kLeg = 16, kPad = 24, kTime = 36;  // first words (row: 0)
+  static constexpr int kLane = 60;     // 56 words; an odd number of 16-byte units
+  static constexpr int kPitch = kEncRound + 1;
+  uint32_t buf[2][32 * kLane];
+  uint32_t res[32 * kPitch];   // row difference | sector/leg << 8 | pad residual << 16
+};
+
+// Truth of the clusters [j, j + m) of a track, m <= kEncRound.
+__device__ __forceinline__ void issue_truth(uint32_t* lb, const EncDev& E, uint32_t j, uint32_t m) {
+  cp_windows<2>(lb, E.row + j, E.row + j + m);
+  cp_windows<2>(lb + EncStage::kSec, E.sector + j, E.sector + j + m);
+  cp_windows<2>(lb + EncStage::kLeg, E.leg + j, E.leg + j + m);
+  cp_windows<3>(lb + EncStage::kPad, E.pad + j, E.pad + j + m);
+  cp_windows<5>(lb + EncStage::kTime, E.time + j, E.time + j + m);
+}
+
+}  // namespace
+
+// Writes the headers and the residual streams of the attached clusters.  One
+// lane per track like the decoder, with the truth staged a round ahead and the
+// residuals leaving through shared memory: read and written directly, 13
+// unrelated sectors per lane and step, the walk took 3.25 ms for 200 k tracks
+// (18 M clusters); staged it takes 0.35 ms.
+__global__ void __launch_bounds__(kDecodeThreads, 3)
+    k_track_encode(const EncDev* enc, const FrameDev* frames, PlanDev plan, uint32_t n_tasks) {
+  constexpr int R = kEncRound, P = EncStage::kPitch;
   __shared__ RowGeo geo;
+  extern __shared__ __align__(16) uint32_t s_stage[];
   fill_row_geo(&geo);
   __syncthreads();
-  const int lane = threadIdx.x & 31;
+  EncStage& S = reinterpret_cast<EncStage*>(s_stage)[threadIdx.x >> 5];
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t sq = lane % R, sg = lane / R;
   for (;;) {
     const uint32_t task = next_task(&plan.counters[0]);
     if (task >= n_tasks) break;
@@ -339,49 +397,125 @@ __global__ void __launch_bounds__(256) k_track_encode(const EncDev* enc, const F
     const EncDev& E = enc[f];
     if (*F.status & kStCount) continue;
     const uint32_t idx = (task - plan.pre_warp[f]) * 32u + lane;
-    const bool act = idx < F.n_tracks;
+    uint8_t* __restrict__ rd_o = E.o_row_diff;
+    uint8_t* __restrict__ sld_o = E.o_sld;
+    uint16_t* __restrict__ pr_o = E.o_pad_res;
+    uint32_t* __restrict__ tr_o = E.o_time_res;
     uint32_t st = 0, t = 0, j0 = 0, n = 0;
     Track s;
-    if (act) {
+    if (idx < F.n_tracks) {
       t = F.order[idx];
       j0 = F.track_start[t];
       n = E.ncl[t];
-      const uint32_t r0 = E.row[j0], s0 = E.sector[j0];
-      if (r0 >= (uint32_t)kNRow || s0 >= (uint32_t)kNSec) st |= kStRow;
-      E.o_qpt[t] = E.qpt[t];
-      E.o_ncl[t] = (uint16_t)n;
-      E.o_row[t] = (uint8_t)r0;
-      E.o_slice[t] = (uint8_t)s0;
-      E.o_pad[t] = E.pad[j0];
-      E.o_time[t] = E.time[j0];
-      seed(&geo, s, E.qpt[t], r0, s0 < (uint32_t)kNSec ? s0 : kNSec - 1, E.pad[j0], E.time[j0]);
     }
-    const uint32_t nmax = __reduce_max_sync(0xffffffffu, n);
-    for (uint32_t k = 1; k < nmax; k++) {
-      if (k < n) {
-        const uint32_t d = j0 - t + k - 1;
-        const uint32_t j = j0 + k;
-        const uint32_t r1 = E.row[j], r0 = E.row[j - 1];
-        const int s1 = E.sector[j], s0 = E.sector[j - 1];
-        if (r1 >= (uint32_t)kNRow || s1 >= kNSec) st |= kStRow;
+    const uint32_t dm1 = j0 - t - 1u;  // cluster k >= 1 has difference dm1 + k
+    const uint32_t rounds = (__reduce_max_sync(kFull, n) + R - 1) / R;
+    uint32_t* lb0 = S.buf[0] + lane * EncStage::kLane;
+    uint32_t* lb1 = S.buf[1] + lane * EncStage::kLane;
+    if (n > 0) issue_truth(lb0, E, j0, min(n, (uint32_t)R));
+    cp_commit();
+    // offsets of a round's first cluster in its windows
+    const int o_row = win_off(E.row + j0), o_sec = win_off(E.sector + j0);
+    const int o_leg = win_off(E.leg + j0), o_pad = win_off(E.pad + j0) / 2;
+    const int o_time = win_off(E.time + j0) / 4;
+    uint32_t r0 = 0, s0 = 0, l0 = 0;  // row, sector, leg of the cluster before
+    for (uint32_t r = 0; r < rounds; r++) {
+      const uint32_t k0 = r * R;
+      uint32_t* lb = (r & 1) ? lb1 : lb0;
+      if (r + 1 < rounds) {
+        if (n > k0 + R) issue_truth((r & 1) ? lb0 : lb1, E, j0 + k0 + R, min(n - k0 - R, (uint32_t)R));
+        cp_commit();
+        cp_wait<1>();
+      } else {
+        cp_wait<0>();
+      }
+      const uint8_t* row_b = reinterpret_cast<const uint8_t*>(lb) + o_row;
+      const uint8_t* sec_b = reinterpret_cast<const uint8_t*>(lb + EncStage::kSec) + o_sec;
+      const uint8_t* leg_b = reinterpret_cast<const uint8_t*>(lb + EncStage::kLeg) + o_leg;
+      const uint16_t* pad_b = reinterpret_cast<const uint16_t*>(lb + EncStage::kPad) + o_pad;
+      uint32_t* time_b = lb + EncStage::kTime + o_time;  // becomes the time residual
+      const uint32_t rem = n > k0 ? n - k0 : 0u;
+      uint32_t q0 = 0;
+      if (k0 == 0) {  // the first cluster is stored absolute
+        if (rem > 0) {
+          r0 = row_b[0];
+          s0 = sec_b[0];
+          l0 = leg_b[0];
+          const uint32_t pad = pad_b[0], time = time_b[0];
+          if (r0 >= (uint32_t)kNRow || s0 >= (uint32_t)kNSec) st |= kStRow;
+          const uint8_t qpt = E.qpt[t];
+          E.o_qpt[t] = qpt;
+          E.o_ncl[t] = (uint16_t)n;
+          E.o_row[t] = (uint8_t)r0;
+          E.o_slice[t] = (uint8_t)s0;
+          E.o_pad[t] = (uint16_t)pad;
+          E.o_time[t] = time;
+          seed(&geo, s, qpt, (int)r0, s0 < (uint32_t)kNSec ? (int)s0 : kNSec - 1, pad, time);
+        }
+        q0 = 1;
+      }
+      auto step = [&](uint32_t q) {
+        const uint32_t r1 = row_b[q], s1 = sec_b[q], l1 = leg_b[q];
+        if (r1 >= (uint32_t)kNRow || s1 >= (uint32_t)kNSec) st |= kStRow;
         const uint32_t rd = (r1 - r0) & 255u;
-        const uint32_t legd = E.leg[j] != E.leg[j - 1] ? 1u : 0u;
-        const uint32_t sd = (uint32_t)(((s1 - s0) % kNSec + kNSec) % kNSec);
-        const uint32_t sld = legd * kNSec + sd;
+        const uint32_t sld = (l1 != l0 ? (uint32_t)kNSec : 0u) + (s1 - s0 + 8u * kNSec) % kNSec;
+        r0 = r1;
+        s0 = s1;
+        l0 = l1;
         st |= key_step(s, rd, sld);
         uint32_t ppad, ptime;
         const float4 G = geo.row[s.row];
         propagate_predict(G, s, ppad, ptime);
-        const uint32_t padq = E.pad[j], timeq = E.time[j];
-        E.o_row_diff[d] = (uint8_t)rd;
-        E.o_sld[d] = (uint8_t)sld;
-        E.o_pad_res[d] = (uint16_t)((padq - ppad) & 0xFFFFu);
-        E.o_time_res[d] = timeq - ptime;
+        const uint32_t padq = pad_b[q], timeq = time_b[q];
+        S.res[lane * P + q] = rd | (sld << 8) | ((padq - ppad) << 16);
+        time_b[q] = timeq - ptime;
         update(G, s, padq, timeq);
+      };
+      const bool full = __all_sync(kFull, rem >= (uint32_t)R);
+      if (full) {
+#pragma unroll 1
+        for (uint32_t q = q0; q < (uint32_t)R; q++) step(q);
+      } else {
+#pragma unroll 1
+        for (uint32_t q = q0; q < (uint32_t)R; q++)
+          if (q < rem) step(q);
       }
+      __syncwarp();
+      const uint32_t k = k0 + sq;
+      const uint32_t* bb = (r & 1) ? S.buf[1] : S.buf[0];
+#pragma unroll 8
+      for (int i0 = 0; i0 < 32; i0 += 32 / R) {
+        const uint32_t i = i0 + sg;
+        const uint32_t di = __shfl_sync(kFull, dm1, i) + k;
+        const uint32_t no = __shfl_sync(kFull, n | ((uint32_t)o_time << 16), i);
+        if (k < (no & 0xFFFFu) && k > 0) {
+          const uint32_t a = S.res[i * P + sq];
+          rd_o[di] = (uint8_t)a;
+          sld_o[di] = (uint8_t)(a >> 8);
+          pr_o[di] = (uint16_t)(a >> 16);
+          tr_o[di] = bb[i * EncStage::kLane + EncStage::kTime + (no >> 16) + sq];
+        }
+      }
+      __syncwarp();
     }
-    if (st) atomicOr(F.status, st);
+    st = __reduce_or_sync(kFull, st);
+    if (st && lane == 0) atomicOr(F.status, st);
   }
+}
+
+constexpr int kEncodeSmem = (kDecodeThreads / 32) * (int)sizeof(EncStage);
+
+void launch_track_encode(uint32_t grid, cudaStream_t st, const EncDev* enc, const FrameDev* frames,
+                         PlanDev plan, uint32_t n_tasks) {
+  k_track_encode<<<grid, kDecodeThreads, kEncodeSmem, st>>>(enc, frames, plan, n_tasks);
+}
+
+cudaError_t prepare_track_encode(int* blocks_per_sm) {
+  const cudaError_t e = cudaFuncSetAttribute(
+      k_track_encode, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncodeSmem);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_track_encode,
+                                                       kDecodeThreads, kEncodeSmem);
 }
 
 }  // namespace tmd

@@ -176,8 +176,9 @@ void launch_unatt_decode(int variant, uint32_t grid, cudaStream_t st, const Fram
                          PlanDev plan, uint32_t n_tickets);
 cudaError_t occupancy_unatt_decode(int* blocks_per_sm);
 __global__ void k_selftest_wait(const unsigned long long* never, uint32_t* status);
-__global__ void k_track_encode(const EncDev* enc, const FrameDev* frames, PlanDev plan,
-                               uint32_t n_tasks);
+void launch_track_encode(uint32_t grid, cudaStream_t st, const EncDev* enc, const FrameDev* frames,
+                         PlanDev plan, uint32_t n_tasks);
+cudaError_t prepare_track_encode(int* blocks_per_sm);
 __global__ void k_track_trace(const FrameDev* frames, const uint32_t* ids, uint32_t n_ids,
                               float* state);
 
