@@ -245,8 +245,8 @@ extern "C" int tmd_create(const tmd_config* cfg, tmd_handle** out) {
                            "event")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_count_rank(), "smem attribute")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_unatt_encode(&h->occ_ue), "unattached encoder")) != TMD_OK ||
-      (rc = tmd_cuda_check(h, occupancy_track_decode(0, &h->occ_decode_v[0]), "occupancy")) != TMD_OK ||
-      (rc = tmd_cuda_check(h, occupancy_track_decode(1, &h->occ_decode_v[1]), "occupancy")) != TMD_OK ||
+      (rc = tmd_cuda_check(h, prepare_track_decode(0, &h->occ_decode_v[0]), "occupancy")) != TMD_OK ||
+      (rc = tmd_cuda_check(h, prepare_track_decode(1, &h->occ_decode_v[1]), "occupancy")) != TMD_OK ||
       (rc = tmd_cuda_check(h, occupancy_unatt_decode(&h->occ_unatt), "occupancy")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_track_encode(&h->occ_encode), "occupancy")) != TMD_OK) {
     delete h;

@@ -51,44 +51,70 @@ constexpr uint32_t kFull = 0xffffffffu;
 
 // ---------------------------------------------------------------------------
 // Asynchronous staging.  Each lane copies its own track's next round of
-// differences into its own part of a double buffer with cp.async (4-byte
-// copies of the aligned words that hold the round's elements, which lie in
-// the caller's allocation), so the copies of round r + 1 are in flight while
-// the lane runs the model through round r, and no lane waits for another
-// lane's copies.  The round's outputs still leave through shared memory with
-// coalesced stores.
+// differences into its own part of a double buffer with cp.async, so the
+// copies of round r + 1 are in flight while the lane runs the model through
+// round r, and no lane waits for another lane's copies.  The round's outputs
+// still leave through shared memory with coalesced stores.
+//
+// A copy moves one 16-byte aligned window (it lies in the same 16 bytes as an
+// element of the caller's array).  Every lane's copy is its own L1 request,
+// and the requests, not the bytes, are what staging costs: a round of 16 steps
+// takes 12 copies per lane (2 + 2 + 3 + 5) where copies of the aligned 4-byte
+// words took 35 (431 -> 407 us for the 37.8 M clusters of a
+// Pb-Pb-shaped frame).
+// ---------------------------------------------------------------------------
 namespace {
 
-__device__ __forceinline__ void cp_word(const uint32_t* dst_smem, uintptr_t src) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst_smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
-}
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// Words per lane and buffer: row_diff and sld (R bytes at any alignment),
-// pad_res (R u16 at any 2-byte alignment), time_res (R words, one per step).
+// Copies the 16-byte windows from the one that holds `first` up to byte `end`
+// (at most W of them).
+template <int W>
+__device__ __forceinline__ void cp_windows(const uint32_t* dst_smem, const void* first,
+                                           const void* end) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst_smem);
+  const uintptr_t w = reinterpret_cast<uintptr_t>(first) & ~(uintptr_t)15;
+  const uintptr_t e = reinterpret_cast<uintptr_t>(end);
+#pragma unroll
+  for (int c = 0; c < W; c++)
+    if (w + 16 * c < e)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d + 16 * c), "l"(w + 16 * c)
+                   : "memory");
+}
+
+// Offset of a byte in its window.
+__device__ __forceinline__ int win_off(const void* p) {
+  return (int)(reinterpret_cast<uintptr_t>(p) & 15);
+}
+
+// Windows that R elements of `size` bytes can touch.
+constexpr int windows(int R, int size) { return (16 - size + R * size + 15) / 16; }
+
+// Words per lane and buffer: windows of row_diff, sld, pad_res and time_res.
 template <int R>
 struct AsyncLayout {
-  static constexpr int kRd = R / 4 + 1;
-  static constexpr int kPr = R / 2 + 1;
-  static constexpr int kTr0 = 2 * kRd + kPr;   // first time_res word
-  static constexpr int kLane = kTr0 + R;       // odd: lanes hit distinct banks
+  static constexpr int kW1 = windows(R, 1), kW2 = windows(R, 2), kW4 = windows(R, 4);
+  static constexpr int kSl = 4 * kW1, kPr = 8 * kW1, kTr = kPr + 4 * kW2;
+  static constexpr int kWin = 2 * kW1 + kW2 + kW4;
+  static constexpr int kLane = 4 * (kWin | 1);  // an odd number of windows: the lanes' 16-byte
+                                                // parts spread over the banks
 };
 
 template <int R>
 struct AsyncStage {
   uint32_t buf[2][32 * AsyncLayout<R>::kLane];
-  uint32_t kp[32 * (R + 1)];  // outputs key | pad << 16 of the round
+  uint32_t kp[32 * (R + 1)];  // outputs key | pad << 16 of the round; [R]: the first
+                              // cluster's time code
 };
 
-// Element offsets of step 0 of a round inside a lane's buffer (negative in
-// round 0, whose step 0 has no difference).
+// Element offsets of step 0 of a round inside a lane's windows (one before
+// the first element in round 0, whose step 0 has no difference).
 struct RoundBase {
-  int rd, sl, pr;
+  int rd, sl, pr, tr;
 };
 
 // Issue the copies of the differences of steps [k0, k0 + R) of one track
@@ -99,44 +125,17 @@ __device__ __forceinline__ RoundBase issue_round(uint32_t* lb, uint32_t k0, uint
                                                  const uint8_t* sld_s, const uint16_t* pr_s,
                                                  const uint32_t* tr_s) {
   using Lay = AsyncLayout<R>;
-  RoundBase rb{0, 0, 0};
   const uint32_t k_lo = k0 > 1u ? k0 : 1u;
   const uint32_t k_hi = k0 + R < n ? k0 + R : n;
-  if (k_lo >= k_hi) return rb;
+  if (k_lo >= k_hi) return RoundBase{0, 0, 0, 0};
   const uint32_t x_lo = dm1 + k_lo, x_hi = dm1 + k_hi;  // differences [x_lo, x_hi)
   const int skip = (int)(k_lo - k0);                    // 1 in round 0, else 0
-  {
-    const uintptr_t a = reinterpret_cast<uintptr_t>(rd_s + x_lo);
-    const uintptr_t e = reinterpret_cast<uintptr_t>(rd_s + x_hi);
-    const uintptr_t w = a & ~(uintptr_t)3;
-#pragma unroll
-    for (int c = 0; c < Lay::kRd; c++)
-      if (w + 4 * c < e) cp_word(lb + c, w + 4 * c);
-    rb.rd = (int)(a - w) - skip;
-  }
-  {
-    const uintptr_t a = reinterpret_cast<uintptr_t>(sld_s + x_lo);
-    const uintptr_t e = reinterpret_cast<uintptr_t>(sld_s + x_hi);
-    const uintptr_t w = a & ~(uintptr_t)3;
-#pragma unroll
-    for (int c = 0; c < Lay::kRd; c++)
-      if (w + 4 * c < e) cp_word(lb + Lay::kRd + c, w + 4 * c);
-    rb.sl = (int)(a - w) - skip;
-  }
-  {
-    const uintptr_t a = reinterpret_cast<uintptr_t>(pr_s + x_lo);
-    const uintptr_t e = reinterpret_cast<uintptr_t>(pr_s + x_hi);
-    const uintptr_t w = a & ~(uintptr_t)3;
-#pragma unroll
-    for (int c = 0; c < Lay::kPr; c++)
-      if (w + 4 * c < e) cp_word(lb + 2 * Lay::kRd + c, w + 4 * c);
-    rb.pr = (int)((a - w) >> 1) - skip;
-  }
-#pragma unroll
-  for (int c = 0; c < R; c++)
-    if (x_lo + c < x_hi)
-      cp_word(lb + Lay::kTr0 + skip + c, reinterpret_cast<uintptr_t>(tr_s + x_lo + c));
-  return rb;
+  cp_windows<Lay::kW1>(lb, rd_s + x_lo, rd_s + x_hi);
+  cp_windows<Lay::kW1>(lb + Lay::kSl, sld_s + x_lo, sld_s + x_hi);
+  cp_windows<Lay::kW2>(lb + Lay::kPr, pr_s + x_lo, pr_s + x_hi);
+  cp_windows<Lay::kW4>(lb + Lay::kTr, tr_s + x_lo, tr_s + x_hi);
+  return RoundBase{win_off(rd_s + x_lo) - skip, win_off(sld_s + x_lo) - skip,
+                   win_off(pr_s + x_lo) / 2 - skip, win_off(tr_s + x_lo) / 4 - skip};
 }
 
 }  // namespace
@@ -151,13 +150,13 @@ __global__ void __launch_bounds__(kDecodeThreads, MINB)
   constexpr int P = R + 1;   // pitch of the output rows
   constexpr int G = 32 / R;  // tracks per write-out instruction
   __shared__ RowGeo geo_s;
-  __shared__ AsyncStage<R> stage[kDecodeThreads / 32];
+  extern __shared__ __align__(16) uint32_t s_stage[];
   fill_row_geo(&geo_s);
   __syncthreads();
   const RowGeo* geo = &geo_s;
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t sq = lane % R, sg = lane / R;
-  AsyncStage<R>& S = stage[threadIdx.x >> 5];
+  AsyncStage<R>& S = reinterpret_cast<AsyncStage<R>*>(s_stage)[threadIdx.x >> 5];
   for (;;) {
     const uint32_t task = next_task(&plan.counters[0]);
     if (task >= n_tasks) break;
@@ -172,8 +171,9 @@ __global__ void __launch_bounds__(kDecodeThreads, MINB)
     uint16_t* __restrict__ key_o = F.keys;
     uint16_t* __restrict__ pad_o = F.kf_pad;
     uint32_t* __restrict__ time_o = F.kf_time;
-    uint32_t j0 = 0, n = 0, dm1 = 0, pad0 = 0, time0 = 0, st = 0;
+    uint32_t j0 = 0, n = 0, dm1 = 0, pad0 = 0, time0 = 0, st = 0, tmax = 0;
     Track s;
+    s.max_row = 0;
     if (idx < F.n_tracks) {
       const uint32_t t = F.order[idx];
       j0 = F.track_start[t];
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(kDecodeThreads, MINB)
     for (uint32_t r = 0; r < n_rounds; r++) {
       const uint32_t k0 = r * R;
       uint32_t* lb = (r & 1) ? lb1 : lb0;
-      RoundBase nxt{0, 0, 0};
+      RoundBase nxt{0, 0, 0, 0};
       if (r + 1 < n_rounds) {
         nxt = issue_round<R>((r & 1) ? lb0 : lb1, k0 + R, n, dm1, rd_s, sld_s, pr_s, tr_s);
         cp_commit();
@@ -208,29 +208,30 @@ __global__ void __launch_bounds__(kDecodeThreads, MINB)
       // buffer (step q at element base + q of each stream; the base is -1 in
       // round 0, whose step 0 reads none)
       const uint8_t* rd_b = reinterpret_cast<const uint8_t*>(lb);
-      const uint8_t* sl_b = reinterpret_cast<const uint8_t*>(lb + Lay::kRd);
-      const uint16_t* pr_b = reinterpret_cast<const uint16_t*>(lb + 2 * Lay::kRd);
+      const uint8_t* sl_b = reinterpret_cast<const uint8_t*>(lb + Lay::kSl);
+      const uint16_t* pr_b = reinterpret_cast<const uint16_t*>(lb + Lay::kPr);
+      uint32_t* tr_b = lb + Lay::kTr + cur.tr;  // becomes the time code
       // one model step: cluster k0 + q >= 1 of the lane's track
       auto step = [&](uint32_t q) {
         const uint32_t rdv = rd_b[cur.rd + (int)q], slv = sl_b[cur.sl + (int)q],
                        prv = pr_b[cur.pr + (int)q];
-        st |= key_step(s, rdv, slv);
+        key_step(geo, s, rdv, slv);
         uint32_t ppad, ptime;
         const float4 G = geo->row[s.row];
         propagate_predict(G, s, ppad, ptime);
         const uint32_t padq = (ppad + prv) & 0xFFFFu;
-        const uint32_t timeq = ptime + lb[Lay::kTr0 + q];
+        const uint32_t timeq = ptime + tr_b[q];
         update(G, s, padq, timeq);
-        if (timeq > 0xFFFFFFu) st |= kStTime;
+        tmax = max(tmax, timeq);
         S.kp[lane * P + q] = (uint32_t)(s.sec * kNRow + s.row) | (padq << 16);
-        lb[Lay::kTr0 + q] = timeq;
+        tr_b[q] = timeq;
       };
       uint32_t q0 = 0;
       if (k0 == 0) {  // the track's first cluster, stored absolute
         if (rem > 0) {
-          if (time0 > 0xFFFFFFu) st |= kStTime;
+          tmax = max(tmax, time0);
           S.kp[lane * P] = (uint32_t)(s.sec * kNRow + s.row) | (pad0 << 16);
-          lb[Lay::kTr0] = time0;
+          S.kp[lane * P + R] = time0;
         }
         q0 = 1;
       }
@@ -238,7 +239,7 @@ __global__ void __launch_bounds__(kDecodeThreads, MINB)
       // per-step bound test (the common case for the long tracks decoded first)
       const bool full = __all_sync(kFull, rem >= (uint32_t)R);
       if (full) {
-#pragma unroll 1
+#pragma unroll 4
         for (uint32_t q = q0; q < (uint32_t)R; q++) step(q);
       } else {
 #pragma unroll 1
@@ -247,45 +248,51 @@ __global__ void __launch_bounds__(kDecodeThreads, MINB)
       }
       __syncwarp();
       const uint32_t k = k0 + sq;
-      const uint32_t* bb = (r & 1) ? S.buf[1] : S.buf[0];
+      const uint32_t* bb = ((r & 1) ? S.buf[1] : S.buf[0]) + Lay::kTr + (int)sq - 1;
 #pragma unroll
       for (int i0 = 0; i0 < 32; i0 += G) {
         const uint32_t i = i0 + sg;
         const uint32_t ji = __shfl_sync(kFull, j0, i);
-        // in a full round every track has step k; otherwise test its length
-        const uint32_t ni = full ? 0xFFFFFFFFu : __shfl_sync(kFull, n, i);
-        if (k < ni) {
+        // length and time offset of track i; in a full round every track has step k
+        const uint32_t no = __shfl_sync(kFull, n | ((uint32_t)(cur.tr + 1) << 16), i);
+        if (full || k < (no & 0xFFFFu)) {
           const uint32_t a = S.kp[i * P + sq];
+          const uint32_t* t = k ? bb + i * Lay::kLane + (no >> 16) : S.kp + i * P + R;
           key_o[ji + k] = (uint16_t)(a & 0xFFFFu);
           pad_o[ji + k] = (uint16_t)(a >> 16);
-          time_o[ji + k] = bb[i * Lay::kLane + Lay::kTr0 + sq];
+          time_o[ji + k] = *t;
         }
       }
 
       __syncwarp();
       cur = nxt;
     }
+    if (s.max_row >= kNRow) st |= kStRow;
+    if (tmax > 0xFFFFFFu) st |= kStTime;
     st = __reduce_or_sync(kFull, st);
     if (st && lane == 0) atomicOr(frames[f].status, st);
   }
 }
 
-// Variants: 0 -> rounds of 16 steps (4 blocks per SM), 1 -> rounds of 8
-// steps (6 blocks per SM).
+template <int R>
+constexpr int kDecodeSmem = (kDecodeThreads / 32) * (int)sizeof(AsyncStage<R>);
+
+// Variants: 0 -> rounds of 16 steps (3 blocks per SM), 1 -> rounds of 8
+// steps (5 blocks per SM).
 void launch_track_decode(int variant, uint32_t grid, cudaStream_t st, const FrameDev* frames,
                          PlanDev plan, uint32_t n_tasks) {
   if (variant == 1)
-    k_track_decode<8, 6><<<grid, kDecodeThreads, 0, st>>>(frames, plan, n_tasks);
+    k_track_decode<8, 5><<<grid, kDecodeThreads, kDecodeSmem<8>, st>>>(frames, plan, n_tasks);
   else
-    k_track_decode<16, 4><<<grid, kDecodeThreads, 0, st>>>(frames, plan, n_tasks);
+    k_track_decode<16, 3><<<grid, kDecodeThreads, kDecodeSmem<16>, st>>>(frames, plan, n_tasks);
 }
 
-cudaError_t occupancy_track_decode(int variant, int* blocks_per_sm) {
-  if (variant == 1)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_track_decode<8, 6>,
-                                                         kDecodeThreads, 0);
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_track_decode<16, 4>,
-                                                       kDecodeThreads, 0);
+cudaError_t prepare_track_decode(int variant, int* blocks_per_sm) {
+  const auto kern = variant == 1 ? k_track_decode<8, 5> : k_track_decode<16, 3>;
+  const int smem = variant == 1 ? kDecodeSmem<8> : kDecodeSmem<16>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, kDecodeThreads, smem);
 }
 
 // Float-path trace: one thread per selected track walks it through the
@@ -311,7 +318,7 @@ __global__ void k_track_trace(const FrameDev* frames, const uint32_t* ids, uint3
   for (uint32_t k = 0; k < n && k < (uint32_t)kNRow; k++) {
     if (k > 0) {
       const uint32_t d = dm1 + k;
-      key_step(s, F.row_diff[d], F.sld[d]);
+      key_step(&geo, s, F.row_diff[d], F.sld[d]);
       uint32_t ppad, ptime;
       const float4 G = geo.row[s.row];
       propagate_predict(G, s, ppad, ptime);
@@ -326,34 +333,14 @@ __global__ void k_track_trace(const FrameDev* frames, const uint32_t* ids, uint3
 }
 
 // ---------------------------------------------------------------------------
-// Encoder staging: 14 copies of 16-byte aligned windows per lane and round of
-// 16 clusters (row, sector and leg 2 each, pad 3, time 5).  A round advances every stream by a multiple
+// Encoder staging: 14 windows per lane and round of 16 clusters (row, sector
+// and leg 2 each, pad 3, time 5).  A round advances every stream by a multiple
 // of 16 bytes, so the offset of a round's first cluster in its windows is a
 // constant of the track.
 // ---------------------------------------------------------------------------
 namespace {
 
 constexpr int kEncRound = 16;
-
-// Copies the 16-byte windows from the one that holds `first` up to byte `end`
-// (at most W of them).
-template <int W>
-__device__ __forceinline__ void cp_windows(const uint32_t* dst_smem, const void* first,
-                                           const void* end) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst_smem);
-  const uintptr_t w = reinterpret_cast<uintptr_t>(first) & ~(uintptr_t)15;
-  const uintptr_t e = reinterpret_cast<uintptr_t>(end);
-#pragma unroll
-  for (int c = 0; c < W; c++)
-    if (w + 16 * c < e)
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d + 16 * c), "l"(w + 16 * c)
-                   : "memory");
-}
-
-// Offset of a byte in its window.
-__device__ __forceinline__ int win_off(const void* p) {
-  return (int)(reinterpret_cast<uintptr_t>(p) & 15);
-}
 
 struct EncStage {
   static constexpr int kSec = 8, kLeg = 16, kPad = 24, kTime = 36;  // first words (row: 0)
@@ -363,8 +350,14 @@ struct EncStage {
   uint32_t res[32 * kPitch];   // row difference | sector/leg << 8 | pad residual << 16
 };
 
+struct Truth {
+  const uint8_t *row, *sector, *leg;
+  const uint16_t* pad;
+  const uint32_t* time;
+};
+
 // Truth of the clusters [j, j + m) of a track, m <= kEncRound.
-__device__ __forceinline__ void issue_truth(uint32_t* lb, const EncDev& E, uint32_t j, uint32_t m) {
+__device__ __forceinline__ void issue_truth(uint32_t* lb, const Truth& E, uint32_t j, uint32_t m) {
   cp_windows<2>(lb, E.row + j, E.row + j + m);
   cp_windows<2>(lb + EncStage::kSec, E.sector + j, E.sector + j + m);
   cp_windows<2>(lb + EncStage::kLeg, E.leg + j, E.leg + j + m);
@@ -394,19 +387,21 @@ __global__ void __launch_bounds__(kDecodeThreads, 3)
     if (task >= n_tasks) break;
     const uint32_t f = find_frame(plan.pre_warp, plan.n_frames, task);
     const FrameDev& F = frames[f];
-    const EncDev& E = enc[f];
+    const EncDev& D = enc[f];
     if (*F.status & kStCount) continue;
     const uint32_t idx = (task - plan.pre_warp[f]) * 32u + lane;
-    uint8_t* __restrict__ rd_o = E.o_row_diff;
-    uint8_t* __restrict__ sld_o = E.o_sld;
-    uint16_t* __restrict__ pr_o = E.o_pad_res;
-    uint32_t* __restrict__ tr_o = E.o_time_res;
-    uint32_t st = 0, t = 0, j0 = 0, n = 0;
+    // in registers: stores to the output bytes may alias the descriptor
+    const Truth E{D.row, D.sector, D.leg, D.pad, D.time};
+    uint8_t* __restrict__ rd_o = D.o_row_diff;
+    uint8_t* __restrict__ sld_o = D.o_sld;
+    uint16_t* __restrict__ pr_o = D.o_pad_res;
+    uint32_t* __restrict__ tr_o = D.o_time_res;
+    uint32_t st = 0, t = 0, j0 = 0, n = 0, rmax = 0, smax = 0;
     Track s;
     if (idx < F.n_tracks) {
       t = F.order[idx];
       j0 = F.track_start[t];
-      n = E.ncl[t];
+      n = D.ncl[t];
     }
     const uint32_t dm1 = j0 - t - 1u;  // cluster k >= 1 has difference dm1 + k
     const uint32_t rounds = (__reduce_max_sync(kFull, n) + R - 1) / R;
@@ -442,27 +437,29 @@ __global__ void __launch_bounds__(kDecodeThreads, 3)
           s0 = sec_b[0];
           l0 = leg_b[0];
           const uint32_t pad = pad_b[0], time = time_b[0];
-          if (r0 >= (uint32_t)kNRow || s0 >= (uint32_t)kNSec) st |= kStRow;
-          const uint8_t qpt = E.qpt[t];
-          E.o_qpt[t] = qpt;
-          E.o_ncl[t] = (uint16_t)n;
-          E.o_row[t] = (uint8_t)r0;
-          E.o_slice[t] = (uint8_t)s0;
-          E.o_pad[t] = (uint16_t)pad;
-          E.o_time[t] = time;
+          rmax = r0;
+          smax = s0;
+          const uint8_t qpt = D.qpt[t];
+          D.o_qpt[t] = qpt;
+          D.o_ncl[t] = (uint16_t)n;
+          D.o_row[t] = (uint8_t)r0;
+          D.o_slice[t] = (uint8_t)s0;
+          D.o_pad[t] = (uint16_t)pad;
+          D.o_time[t] = time;
           seed(&geo, s, qpt, (int)r0, s0 < (uint32_t)kNSec ? (int)s0 : kNSec - 1, pad, time);
         }
         q0 = 1;
       }
       auto step = [&](uint32_t q) {
         const uint32_t r1 = row_b[q], s1 = sec_b[q], l1 = leg_b[q];
-        if (r1 >= (uint32_t)kNRow || s1 >= (uint32_t)kNSec) st |= kStRow;
+        rmax = max(rmax, r1);
+        smax = max(smax, s1);
         const uint32_t rd = (r1 - r0) & 255u;
         const uint32_t sld = (l1 != l0 ? (uint32_t)kNSec : 0u) + (s1 - s0 + 8u * kNSec) % kNSec;
         r0 = r1;
         s0 = s1;
         l0 = l1;
-        st |= key_step(s, rd, sld);
+        key_step(&geo, s, rd, sld);
         uint32_t ppad, ptime;
         const float4 G = geo.row[s.row];
         propagate_predict(G, s, ppad, ptime);
@@ -473,7 +470,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 3)
       };
       const bool full = __all_sync(kFull, rem >= (uint32_t)R);
       if (full) {
-#pragma unroll 1
+#pragma unroll 4
         for (uint32_t q = q0; q < (uint32_t)R; q++) step(q);
       } else {
 #pragma unroll 1
@@ -498,6 +495,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 3)
       }
       __syncwarp();
     }
+    if (rmax >= (uint32_t)kNRow || smax >= (uint32_t)kNSec) st |= kStRow;
     st = __reduce_or_sync(kFull, st);
     if (st && lane == 0) atomicOr(F.status, st);
   }

@@ -165,7 +165,7 @@ __global__ void k_tile_base(const FrameDev* frames, PlanDev plan);
 // every attached cluster.
 void launch_track_decode(int variant, uint32_t grid, cudaStream_t st, const FrameDev* frames,
                          PlanDev plan, uint32_t n_tasks);
-cudaError_t occupancy_track_decode(int variant, int* blocks_per_sm);
+cudaError_t prepare_track_decode(int variant, int* blocks_per_sm);
 // Record scatter variants 0, 1 (identical results; see tmd_scatter.cu),
 // launched over n_tiles ranking tiles of all frames.
 void launch_att_scatter(int variant, uint32_t n_tiles, cudaStream_t st, const FrameDev* frames,

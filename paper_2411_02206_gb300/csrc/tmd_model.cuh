@@ -37,6 +37,25 @@ __device__ __forceinline__ float fdiv(float a, float b) { return __fdiv_rn(a, b)
 __device__ __forceinline__ float ffma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 // 1/x correctly rounded: the same value as the division 1.0f / x.
 __device__ __forceinline__ float frcp(float x) { return __frcp_rn(x); }
+// Two correctly rounded reciprocals at once.  The hardware approximation and
+// one correction y + y (1 - x y) (P. Markstein, IBM J. Res. Dev. 34, 1990) give
+// the value of __frcp_rn wherever 1 - x y is small, which was checked on all
+// 2^32 operands; the others (zero, denormal, huge, infinite, NaN) take
+// __frcp_rn.  Two calls of __frcp_rn are two branches that cut a model step
+// into pieces executed one after the other; here one test serves both and the
+// two chains and the code around them interleave.
+__device__ __forceinline__ void frcp2(float a, float b, float& ia, float& ib) {
+  float ya, yb;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ya) : "f"(a));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yb) : "f"(b));
+  const float ea = __fmaf_rn(-a, ya, 1.0f), eb = __fmaf_rn(-b, yb, 1.0f);
+  ia = __fmaf_rn(ya, ea, ya);
+  ib = __fmaf_rn(yb, eb, yb);
+  if (!(__fadd_rn(fabsf(ea), fabsf(eb)) < 0.0009765625f)) {  // also for NaN
+    ia = __frcp_rn(a);
+    ib = __frcp_rn(b);
+  }
+}
 
 // Model constants (binary32).
 constexpr float kSY2 = 0.01f;     // measurement variance of y [cm^2]
@@ -70,6 +89,7 @@ __constant__ float c_sin20[18] = {
 // with a single shared-memory load.
 struct RowGeo {
   float4 row[kNRow];
+  float2 rot[18];  // cos, sin of k * 20 deg: lanes change sector by different k
 };
 
 __device__ __forceinline__ void fill_row_geo(RowGeo* g) {
@@ -78,6 +98,7 @@ __device__ __forceinline__ void fill_row_geo(RowGeo* g) {
     const float x = 85.0f + (float)r;
     const float w = fdiv(fmul(fmul(2.0f, x), kTan10), (float)np);
     g->row[r] = make_float4(x, w, fdiv(1.0f, w), fmul(0.5f, (float)np));
+    if (r < 18) g->rot[r] = make_float2(c_cos20[r], c_sin20[r]);
   }
 }
 
@@ -95,6 +116,7 @@ struct Track {
   float c00, c01, c02, c11, c12, c22;
   float t, tt, d00, d01, d11;
   int raw_row;  // row accumulator (mod 256); the model uses min(raw_row, 151)
+  int max_row;  // largest raw_row reached by a step
   int row;
   int sec;
 };
@@ -119,6 +141,7 @@ __device__ __forceinline__ void seed(const RowGeo* g, Track& s, uint8_t qpta, in
                                      int sec, uint32_t padq, uint32_t timeq) {
   const float qpt = fmul(fsub((float)qpta, 127.5f), 0.078125f);
   s.raw_row = raw_row;
+  s.max_row = 0;
   s.row = raw_row < kNRow ? raw_row : kNRow - 1;
   s.sec = sec;
   const float4 G = g->row[s.row];
@@ -142,11 +165,14 @@ __device__ __forceinline__ void leg_change(Track& s) {
   reset_ycov(s);
 }
 
-// Sector change to nsec: rotate the parabola's point, slope and curvature by
-// k * 20 deg; a change of side (A/C) reverses the time slope.
-__device__ __forceinline__ void sector_change(Track& s, int nsec) {
-  const int k = ((nsec % 18) - (s.sec % 18) + 18) % 18;
-  const float ca = c_cos20[k], sa = c_sin20[k];
+// Sector change by sd = 1..35 sectors (mod 36): rotate the parabola's point,
+// slope and curvature by sd * 20 deg; a change of side (A/C) reverses the time
+// slope.
+__device__ __forceinline__ void sector_change(const RowGeo* g, Track& s, int sd) {
+  int nsec = s.sec + sd;
+  nsec = nsec >= kNSec ? nsec - kNSec : nsec;
+  const float2 cs = g->rot[sd >= 18 ? sd - 18 : sd];
+  const float ca = cs.x, sa = cs.y;
   float a = fadd(ca, fmul(s.ty, sa));
   const float b = fsub(fmul(s.ty, ca), sa);
   if (!(a >= 1.0e-3f || a <= -1.0e-3f)) a = (a < 0.0f) ? -1.0e-3f : 1.0e-3f;
@@ -165,22 +191,21 @@ __device__ __forceinline__ void sector_change(Track& s, int nsec) {
   reset_ycov(s);
 }
 
-// Key step of one cluster: row and sector/leg differences.  Returns kStRow if
-// the row left the detector.
-__device__ __forceinline__ uint32_t key_step(Track& s, uint32_t row_diff, uint32_t sld) {
-  const uint32_t leg = sld / kNSec;
-  const uint32_t sd = sld - leg * kNSec;
+// Key step of one cluster: row and sector/leg differences.  A row outside the
+// detector shows in s.max_row.
+__device__ __forceinline__ void key_step(const RowGeo* g, Track& s, uint32_t row_diff,
+                                         uint32_t sld) {
   s.raw_row = (s.raw_row + (int)row_diff) & 255;
-  uint32_t st = 0;
-  s.row = s.raw_row;
-  if (s.row >= kNRow) { st = kStRow; s.row = kNRow - 1; }
-  if (leg != 0) leg_change(s);
-  if (sd != 0) {
-    int ns = s.sec + (int)sd;
-    ns = ns >= kNSec ? ns - kNSec : ns;
-    sector_change(s, ns);
+  s.max_row = max(s.max_row, s.raw_row);
+  s.row = min(s.raw_row, kNRow - 1);
+  if (sld != 0) {  // few clusters
+    uint32_t sd = sld;
+    if (sld >= (uint32_t)kNSec) {
+      leg_change(s);
+      sd = sld % kNSec;
+    }
+    if (sd != 0) sector_change(g, s, (int)sd);
   }
-  return st;
 }
 
 // Propagate to the plane of the current row, whose geometry is
@@ -221,7 +246,8 @@ __device__ __forceinline__ void propagate_predict(const float4& G, Track& s, uin
 __device__ __forceinline__ void update(const float4& G, Track& s, uint32_t padq, uint32_t timeq) {
   const float ym = pad_to_y(G, padq);
   const float tm = time_to_t(timeq);
-  const float inv = frcp(fadd(s.c00, kSY2));
+  float inv, invt;
+  frcp2(fadd(s.c00, kSY2), fadd(s.d00, kST2), inv, invt);
   const float k0 = fmul(s.c00, inv), k1 = fmul(s.c01, inv), k2 = fmul(s.c02, inv);
   const float r = fsub(ym, s.y);
   s.y = ffma(k0, r, s.y);
@@ -234,7 +260,6 @@ __device__ __forceinline__ void update(const float4& G, Track& s, uint32_t padq,
   s.c11 = ffma(-k1, c01, s.c11);
   s.c12 = ffma(-k1, c02, s.c12);
   s.c22 = ffma(-k2, c02, s.c22);
-  const float invt = frcp(fadd(s.d00, kST2));
   const float g0 = fmul(s.d00, invt), g1 = fmul(s.d01, invt);
   const float rt = fsub(tm, s.t);
   s.t = ffma(g0, rt, s.t);

@@ -106,7 +106,7 @@ extern "C" int tmd_decode_frame_noalloc(const tmd_frame_in* in, const tmd_frame_
       int sms = 0, od = 0, ou = 0;
       if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
           prepare_count_rank() != cudaSuccess ||
-          occupancy_track_decode(0, &od) != cudaSuccess ||
+          prepare_track_decode(0, &od) != cudaSuccess ||
           occupancy_unatt_decode(&ou) != cudaSuccess) {
         set_err(err, err_len, "device set-up failed");
         return TMD_ERR_CUDA;
