@@ -29,8 +29,8 @@
 // wide between the bin's first and last time, so a bucket holds about one
 // cluster and a few comparisons finish it.  The previous form, eight stable
 // radix passes over 64-bit keys and a random gather of the charges, moved each
-// cluster nine times: 3.60 ms for 20 M clusters against 0.72 ms now, and 0.193 ms
-// in 35 launches for 100 k clusters against 0.058 ms in 8.
+// cluster nine times: 3.60 ms for 20 M clusters against 0.59 ms now, and 0.193 ms
+// in 35 launches for 100 k clusters against 0.054 ms in 8.
 #include <algorithm>
 #include <cstring>
 
@@ -196,61 +196,72 @@ __global__ void __launch_bounds__(1024) k_ue_plan(UeArgs a, UePlan* plan, UeCtl*
 
 // Records to their bins.  A block counts its clusters per bin in shared memory
 // (each cluster's count is its place among the block's clusters of the bin),
-// reserves the bins' ranges with one global atomic per bin, all in flight
-// together, and writes 16-byte records.  The order within a bin depends on the
-// blocks' timing; the sort does not, because the record carries the input index.
-// Larger tiles (G groups of four clusters per thread) reserve less often and
-// write longer runs; small frames take small tiles to occupy every SM.
-template <int G>
-__global__ void __launch_bounds__(kUeScatThreads, 2) k_ue_scatter(UeArgs a, uint4* __restrict__ rec,
+// reserves the bins' ranges with one global atomic per bin, neighbouring bins
+// by neighbouring lanes, and writes 16-byte records.  The order within a bin
+// depends on the blocks' timing; the sort does not, because the record carries
+// the input index.  Bound by L2 requests, of which every record is one.  Small
+// tiles are best although they reserve more often: the records in flight have
+// to meet their neighbours of a sector in L2, and tiles of 16384 spilled
+// half-written sectors (427 us for 20 M clusters against 295 us with 2048).
+// Reserving by the first cluster of each bin, without the pass over the
+// counters, makes every reservation a request of its own: 442 us.
+__global__ void __launch_bounds__(kUeScatThreads, 3) k_ue_scatter(UeArgs a, uint4* __restrict__ rec,
                                                                  UePlan* plan, UeCtl* ctl) {
   constexpr int T = kUeScatThreads;
-  constexpr int Q = (kNBin + T - 1) / T;
-  __shared__ uint32_t s_cnt[kNBin];
+  __shared__ __align__(16) uint32_t s_cnt[kNBin];
   const uint32_t tid = threadIdx.x;
-  for (int i = tid; i < kNBin; i += T) s_cnt[i] = 0u;
-  __syncthreads();
-  const uint32_t base = blockIdx.x * (uint32_t)(T * 4 * G);
-  const uint32_t cnt = min((uint32_t)(T * 4 * G), a.n - base);
-  uint32_t kr[4 * G];  // bin | place in the block's clusters of the bin << 13
-  uint32_t st = 0;
+  const uint32_t base = blockIdx.x * (uint32_t)(T * 4);
+  const uint32_t cnt = min((uint32_t)(T * 4), a.n - base);
+  const uint32_t l = tid * 4, i = base + l;
+  const bool vec = a.vec && l + 4 <= cnt;
+  uint32_t r = 0, s = 0, tm[4] = {}, pd[4] = {}, qt[4] = {}, qm[4] = {}, fl = 0, sp = 0, sg = 0;
+  if (vec) {
+    r = *reinterpret_cast<const uint32_t*>(a.row + i);
+    s = *reinterpret_cast<const uint32_t*>(a.sector + i);
+    const uint4 t = *reinterpret_cast<const uint4*>(a.time + i);
+    const uint2 p = *reinterpret_cast<const uint2*>(a.pad + i);
+    const uint2 x = *reinterpret_cast<const uint2*>(a.qtot + i);
+    const uint2 y = *reinterpret_cast<const uint2*>(a.qmax + i);
+    fl = *reinterpret_cast<const uint32_t*>(a.flags + i);
+    sp = *reinterpret_cast<const uint32_t*>(a.sigp + i);
+    sg = *reinterpret_cast<const uint32_t*>(a.sigt + i);
+    tm[0] = t.x; tm[1] = t.y; tm[2] = t.z; tm[3] = t.w;
+    pd[0] = p.x & 0xFFFFu; pd[1] = p.x >> 16; pd[2] = p.y & 0xFFFFu; pd[3] = p.y >> 16;
+    qt[0] = x.x & 0xFFFFu; qt[1] = x.x >> 16; qt[2] = x.y & 0xFFFFu; qt[3] = x.y >> 16;
+    qm[0] = y.x & 0xFFFFu; qm[1] = y.x >> 16; qm[2] = y.y & 0xFFFFu; qm[3] = y.y >> 16;
+  } else {
 #pragma unroll
-  for (int g = 0; g < G; g++) {
-    const uint32_t l = (g * T + tid) * 4;
-    uint32_t r = 0, s = 0;
-    if (a.vec && l + 4 <= cnt) {
-      r = *reinterpret_cast<const uint32_t*>(a.row + base + l);
-      s = *reinterpret_cast<const uint32_t*>(a.sector + base + l);
-    } else {
-#pragma unroll
-      for (int q = 0; q < 4; q++)
-        if (l + q < cnt) {
-          r |= (uint32_t)a.row[base + l + q] << (8 * q);
-          s |= (uint32_t)a.sector[base + l + q] << (8 * q);
-        }
-    }
-    kr[4 * g] = r;  // row and sector bytes until they are counted
-    kr[4 * g + 1] = s;
-  }
-#pragma unroll
-  for (int g = 0; g < G; g++) {
-    const uint32_t l = (g * T + tid) * 4, r = kr[4 * g], s = kr[4 * g + 1];
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-      kr[4 * g + q] = 0xFFFFFFFFu;
+    for (int q = 0; q < 4; q++)
       if (l + q < cnt) {
-        const uint32_t b = ue_bin((r >> (8 * q)) & 255u, (s >> (8 * q)) & 255u, st);
-        kr[4 * g + q] = b | (atomicAdd(&s_cnt[b], 1u) << 13);
+        r |= (uint32_t)a.row[i + q] << (8 * q);
+        s |= (uint32_t)a.sector[i + q] << (8 * q);
+        tm[q] = a.time[i + q];
+        pd[q] = a.pad[i + q];
+        qt[q] = a.qtot[i + q];
+        qm[q] = a.qmax[i + q];
+        fl |= (uint32_t)a.flags[i + q] << (8 * q);
+        sp |= (uint32_t)a.sigp[i + q] << (8 * q);
+        sg |= (uint32_t)a.sigt[i + q] << (8 * q);
       }
-    }
+  }
+  static_assert(kNBin % 4 == 0, "");
+  for (int z = tid; z < kNBin / 4; z += T)
+    reinterpret_cast<uint4*>(s_cnt)[z] = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
+  uint32_t b[4], place[4], st = 0;
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    b[q] = ue_bin((r >> (8 * q)) & 255u, (s >> (8 * q)) & 255u, st);
+    place[q] = l + q < cnt ? atomicAdd(&s_cnt[b[q]], 1u) : 0u;
   }
   __syncthreads();
+  constexpr int Q = (kNBin + T - 1) / T;
   uint32_t c[Q];
 #pragma unroll
   for (int q = 0; q < Q; q++) {
-    const uint32_t b = tid + q * T;
-    c[q] = b < (uint32_t)kNBin ? s_cnt[b] : 0u;
-    if (c[q]) c[q] = atomicAdd(&plan->cursor[b], c[q]);
+    const uint32_t k = tid + q * T;
+    c[q] = k < (uint32_t)kNBin ? s_cnt[k] : 0u;
+    if (c[q]) c[q] = atomicAdd(&plan->cursor[k], c[q]);
   }
 #pragma unroll
   for (int q = 0; q < Q; q++)
@@ -258,45 +269,14 @@ __global__ void __launch_bounds__(kUeScatThreads, 2) k_ue_scatter(UeArgs a, uint
   __syncthreads();
   bool wide = false;
 #pragma unroll
-  for (int g = 0; g < G; g++) {
-    const uint32_t l = (g * T + tid) * 4, i = base + l;
-    uint32_t tm[4] = {}, pd[4] = {}, qt[4] = {}, qm[4] = {}, fl = 0, sp = 0, sg = 0;
-    if (a.vec && l + 4 <= cnt) {
-      const uint4 t = *reinterpret_cast<const uint4*>(a.time + i);
-      const uint2 p = *reinterpret_cast<const uint2*>(a.pad + i);
-      const uint2 x = *reinterpret_cast<const uint2*>(a.qtot + i);
-      const uint2 y = *reinterpret_cast<const uint2*>(a.qmax + i);
-      fl = *reinterpret_cast<const uint32_t*>(a.flags + i);
-      sp = *reinterpret_cast<const uint32_t*>(a.sigp + i);
-      sg = *reinterpret_cast<const uint32_t*>(a.sigt + i);
-      tm[0] = t.x; tm[1] = t.y; tm[2] = t.z; tm[3] = t.w;
-      pd[0] = p.x & 0xFFFFu; pd[1] = p.x >> 16; pd[2] = p.y & 0xFFFFu; pd[3] = p.y >> 16;
-      qt[0] = x.x & 0xFFFFu; qt[1] = x.x >> 16; qt[2] = x.y & 0xFFFFu; qt[3] = x.y >> 16;
-      qm[0] = y.x & 0xFFFFu; qm[1] = y.x >> 16; qm[2] = y.y & 0xFFFFu; qm[3] = y.y >> 16;
-    } else {
-#pragma unroll
-      for (int q = 0; q < 4; q++)
-        if (l + q < cnt) {
-          tm[q] = a.time[i + q];
-          pd[q] = a.pad[i + q];
-          qt[q] = a.qtot[i + q];
-          qm[q] = a.qmax[i + q];
-          fl |= (uint32_t)a.flags[i + q] << (8 * q);
-          sp |= (uint32_t)a.sigp[i + q] << (8 * q);
-          sg |= (uint32_t)a.sigt[i + q] << (8 * q);
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-      const uint32_t k = kr[4 * g + q];
-      if (k == 0xFFFFFFFFu) continue;
+  for (int q = 0; q < 4; q++)
+    if (l + q < cnt) {
       wide |= (tm[q] >> 24) != 0;
-      rec[s_cnt[k & 8191u] + (k >> 13)] =
+      rec[s_cnt[b[q]] + place[q]] =
           make_uint4((tm[q] & 0xFFFFFFu) | ((fl >> (8 * q)) << 24),
                      pd[q] | (((sg >> (8 * q)) & 255u) << 16) | ((sp >> (8 * q)) << 24),
                      qm[q] | (qt[q] << 16), i + q);
     }
-  }
   if (__syncthreads_or(wide) && tid == 0) ctl->wide = 1u;
 }
 
@@ -866,14 +846,8 @@ extern "C" int tmd_encode_unattached(tmd_handle* h, const tmd_unatt_truth_in* in
   if (n) {
     k_ue_count<<<std::min(2 * sms, n / 8192 + 1), 1024, 0, st>>>(a);
     k_ue_plan<<<1, 1024, 0, st>>>(a, plan, ctl);
-    // the largest tile that still gives every SM two blocks
-    auto tiles = [n](uint32_t g) { return n / (kUeScatThreads * 4 * g) + (n % (kUeScatThreads * 4 * g) != 0); };
-    if (tiles(8) >= 2 * sms)
-      k_ue_scatter<8><<<tiles(8), kUeScatThreads, 0, st>>>(a, r0, plan, ctl);
-    else if (tiles(2) >= 2 * sms)
-      k_ue_scatter<2><<<tiles(2), kUeScatThreads, 0, st>>>(a, r0, plan, ctl);
-    else
-      k_ue_scatter<1><<<tiles(1), kUeScatThreads, 0, st>>>(a, r0, plan, ctl);
+    k_ue_scatter<<<n / (kUeScatThreads * 4) + (n % (kUeScatThreads * 4) != 0), kUeScatThreads, 0,
+                   st>>>(a, r0, plan, ctl);
     k_ue_sort_warp<<<(kNBin + 7) / 8, 256, 0, st>>>(a, r0, plan, ctl);
     if (n > kUeWarpMax)
       k_ue_sort_block<<<std::min(3 * sms, n / kUeWarpMax), kUeBlockThreads, kUeBlockSmem, st>>>(
