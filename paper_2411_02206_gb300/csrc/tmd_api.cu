@@ -244,6 +244,7 @@ extern "C" int tmd_create(const tmd_config* cfg, tmd_handle** out) {
       (rc = tmd_cuda_check(h, cudaEventCreateWithFlags(&h->scratch_done, cudaEventDisableTiming),
                            "event")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_count_rank(), "smem attribute")) != TMD_OK ||
+      (rc = tmd_cuda_check(h, prepare_rans_decode(), "smem attribute")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_unatt_encode(&h->occ_ue), "unattached encoder")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_track_decode(0, &h->occ_decode_v[0]), "occupancy")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_track_decode(1, &h->occ_decode_v[1]), "occupancy")) != TMD_OK ||

@@ -63,7 +63,7 @@ struct tmd_handle {
                                  // (1), after it (0), or by the frames' mix (2)
   int tune_decode_bps = 0;       // decode blocks per SM (0: as many as fit)
   int tune_unatt_bps = 1;        // unattached-decode blocks per SM (0: as many as fit)
-  int tune_rans_overlap = 1;      // 4-byte streams entropy-decoded on the second stream
+  int tune_rans_overlap = 1;      // no effect: all widths are entropy-decoded in one launch
   int tune_coded_overlap = 2;    // coded frames: charges and unattached streams entropy-
                                  // decoded on the second stream beside the track decoder
   cudaEvent_t coded_late = nullptr;   // recorded after those streams are decoded
@@ -146,6 +146,8 @@ int tmd_enqueue(tmd_handle* h, uint32_t nf, const tmd_frame_in* in, const tmd_fr
                 const tmd_truth_in* tin, const tmd_track_out* tout, void* scratch,
                 void* host_record, void* dev_record, cudaStream_t st, bool profile,
                 const ChainStreams* cs = nullptr, const TraceReq* trace = nullptr);
+// Shared-memory attribute of the entropy decoder.
+cudaError_t prepare_rans_decode();
 void tmd_serve_shutdown(tmd_handle* h);
 // Read the tuning parameters for this GPU from the autotune cache, if any.
 void tmd_tune_load(tmd_handle* h);

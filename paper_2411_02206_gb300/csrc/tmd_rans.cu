@@ -12,12 +12,13 @@
 // slot tables in shared memory (slot -> symbol, frequency, offset in one
 // u32), then every lane decodes its stream: per symbol one shared-memory
 // lookup, one multiply-add and, on renormalisation, the next 16-bit word from
-// a two-pair prefetch of the lane's own words (the words of a chunk are
-// interleaved by lane, so a warp's loads of pair j are one 128-byte line).
-// Values are written by the lane at positions 32 k + l: a warp stores 32
-// consecutive values per step.  Three launches, one per value width, size
-// blocks and shared memory for their tables (16, 32, 64 KB); the 4-byte
-// streams run on the handle's second stream beside the others.
+// a queue of the lane's own words that asynchronous copies keep kRing pairs
+// ahead (the words of a chunk are interleaved by lane, so a warp's copies of
+// pair j are one 128-byte line).  Values are written by the lane at positions
+// 32 k + l: a warp stores 32 consecutive values per step.  Streams of all
+// widths share a launch, the widest first: a lane's chain of 256 to 1024
+// dependent symbols takes tens of microseconds whatever the frame's size, and
+// launches of one width after another add those up.
 // tmd_decode_coded_frame entropy-decodes the streams the track decoder and the
 // ranking read first and the attached charges and unattached streams on the
 // second stream while the track decoder runs; the decode chain waits for them
@@ -248,7 +249,9 @@ void encode_stream(const void* vals, uint32_t n, unsigned threads, std::vector<u
 // ---------------------------------------------------------------------------
 // Device decoder
 // ---------------------------------------------------------------------------
-constexpr int kMaxJobFields = 12;
+constexpr int kRing = 4;           // word pairs per lane in flight
+constexpr int kMaxThreads = 512;
+constexpr int kCumWords = 257;     // cumulative frequencies of a plane
 
 struct JobField {
   void* dst;        // decoded values
@@ -256,6 +259,7 @@ struct JobField {
   uint32_t nch;     // chunks
   uint32_t block0;  // first block of this stream in the launch
   uint32_t index;   // directory index
+  uint32_t width;   // bytes per value
 };
 
 struct Job {
@@ -264,7 +268,7 @@ struct Job {
   uint32_t nt, na, nu;
   uint32_t nf;
   uint32_t* status;
-  JobField f[kMaxJobFields];
+  JobField f[kFields];
 };
 
 template <int W> struct ValueType;
@@ -297,18 +301,28 @@ __device__ uint64_t check_entry(const Job& J, const JobField& F, uint32_t w) {
   return off;
 }
 
-// A lane branches into the word refill when its state falls below 2^16 (the
-// warp runs the refill path whenever any lane needs it).
-template <int W, int THREADS, int MINB>
-__global__ void __launch_bounds__(THREADS, MINB) k_rans_decode(const __grid_constant__ Job J) {
+// Copies one word pair to the lane's queue, or zeros if there is none.
+__device__ __forceinline__ void queue_pair(uint32_t* slot, const uint32_t* src, bool some) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(slot);
+  asm volatile(
+      "cp.async.ca.shared.global [%0], [%1], 4, %2;\n\t"
+      "cp.async.commit_group;" ::"r"(d), "l"(src), "r"(some ? 4 : 0) : "memory");
+}
+template <int N>
+__device__ __forceinline__ void queue_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// The chunks of one block, blockDim / 32 of them.  s_tab: W * 4096 slot
+// entries, symbol | (f - 1) << 8 | offset << 20; s_ring: kRing pairs per
+// thread, and before that the cumulative frequencies (kCumWords per plane).
+template <int W>
+__device__ __forceinline__ void decode_block(const Job& J, const JobField& F, uint32_t* s_tab,
+                                             uint32_t* s_ring) {
   using T = typename ValueType<W>::T;
-  extern __shared__ uint32_t s_tab[];  // W * 4096 slot entries: d | sym << 12 | (f - 1) << 20
-  __shared__ uint32_t s_cum[W][257];
+  uint32_t(*s_cum)[kCumWords] = reinterpret_cast<uint32_t(*)[kCumWords]>(s_ring);
   __shared__ uint64_t s_off, s_len;
   __shared__ int s_bad;
-  int fi = 0;
-  while (fi + 1 < (int)J.nf && blockIdx.x >= J.f[fi + 1].block0) fi++;
-  const JobField& F = J.f[fi];
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     const uint64_t off = check_entry(J, F, W);
@@ -341,20 +355,33 @@ __global__ void __launch_bounds__(THREADS, MINB) k_rans_decode(const __grid_cons
   __syncthreads();
   const bool bad_block = s_bad != 0;
   if (!bad_block) {
-    for (uint32_t i = threadIdx.x; i < W * kM; i += THREADS) {
-      const uint32_t p = i >> 12, slot = i & (kM - 1);
-      uint32_t lo = 0, hi = 255;  // largest s with cum[s] <= slot
+    // 8 consecutive slots per thread: one search, then forward
+    for (uint32_t i = threadIdx.x; i < W * kM / 8; i += blockDim.x) {
+      const uint32_t* cum = s_cum[i / (kM / 8)];
+      const uint32_t slot0 = 8 * (i % (kM / 8));
+      uint32_t lo = 0, hi = 255;  // largest s with cum[s] <= slot0
       while (lo < hi) {
         const uint32_t mid = (lo + hi + 1) >> 1;
-        if (s_cum[p][mid] <= slot) lo = mid; else hi = mid - 1;
+        if (cum[mid] <= slot0) lo = mid; else hi = mid - 1;
       }
-      const uint32_t f = s_cum[p][lo + 1] - s_cum[p][lo];
-      s_tab[i] = (slot - s_cum[p][lo]) | (lo << 12) | ((f - 1) << 20);
+      uint32_t c0 = cum[lo], c1 = cum[lo + 1], e[8];
+#pragma unroll
+      for (int k = 0; k < 8; k++) {
+        while (slot0 + k >= c1) {  // cum[256] = 4096 ends every walk
+          lo++;
+          c0 = c1;
+          c1 = cum[lo + 1];
+        }
+        e[k] = lo | ((c1 - c0 - 1) << 8) | ((slot0 + k - c0) << 20);
+      }
+      uint4* t = reinterpret_cast<uint4*>(s_tab) + 2 * i;
+      t[0] = make_uint4(e[0], e[1], e[2], e[3]);
+      t[1] = make_uint4(e[4], e[5], e[6], e[7]);
     }
   }
   __syncthreads();
 
-  const uint32_t chunk = (blockIdx.x - F.block0) * (THREADS / 32) + warp;
+  const uint32_t chunk = (blockIdx.x - F.block0) * (blockDim.x / 32) + warp;
   bool bad = false;
   if (chunk < F.nch) {
     const uint64_t base = (uint64_t)chunk * kChunk + lane;
@@ -373,48 +400,74 @@ __global__ void __launch_bounds__(THREADS, MINB) k_rans_decode(const __grid_cons
       if (w1 < w0 || ((w1 - w0) & 31u) || w1 > slots) bad = true;
       else maxp = (w1 - w0) >> 5;
       const uint32_t* P = reinterpret_cast<const uint32_t*>(sec + a_words) + w0 + lane;
+      uint32_t* ring = s_ring + warp * (32 * kRing) + lane;
+#pragma unroll
+      for (uint32_t i = 0; i < (uint32_t)kRing; i++) {
+        queue_pair(ring + 32 * i, P, i < maxp);
+        P += 32;
+      }
       uint32_t x = st[32ull * chunk + lane];
-      uint32_t cur = maxp > 0 ? __ldg(P) : 0u;
-      uint32_t nxt = maxp > 1 ? __ldg(P + 32) : 0u;
-      uint32_t j = 0;  // pair held in cur
-      bool half = false;
+      queue_wait<kRing - 1>();
+      uint32_t cur = ring[0];  // the next word in its low half
+      uint32_t j = 0;          // pair held in cur
+      bool half = false;       // its first word is used
       for (uint32_t k = 0; k < nk; k++) {
         uint32_t v = 0;
 #pragma unroll
         for (int p = 0; p < W; p++) {
           const uint32_t e = s_tab[p * kM + (x & (kM - 1))];
-          x = ((e >> 20) + 1) * (x >> 12) + (e & (kM - 1));
-          v |= ((e >> 12) & 0xFFu) << (8 * p);
+          const uint32_t xs = x >> 12;
+          x = ((e >> 8) & (kM - 1)) * xs + xs + (e >> 20);
+          v = __byte_perm(v, e, p == 0 ? 0x3214 : p == 1 ? 0x3240 : p == 2 ? 0x3410 : 0x4210);
           if (x < kLower) {
-            if (j >= maxp) bad = true;
-            x = (x << 16) | (half ? cur >> 16 : cur & 0xFFFFu);
+            x = __byte_perm(cur, x, 0x5410);
+            if (x < kLower) bad = true;
+            cur >>= 16;
             if (half) {
-              cur = nxt;
+              queue_pair(ring + 32 * (j % kRing), P, j + kRing < maxp);
+              P += 32;
               j++;
-              nxt = j + 1 < maxp ? __ldg(P + 32ull * (j + 1)) : 0u;
+              queue_wait<kRing - 1>();
+              cur = ring[32 * (j % kRing)];
             }
             half = !half;
-            if (x < kLower) bad = true;
           }
         }
         out[32ull * k] = (T)v;
       }
-      if (x != kLower) bad = true;
+      // every word came from the chunk, and the encoder's start state is left
+      if (2 * j + (half ? 1u : 0u) > 2 * maxp || x != kLower) bad = true;
     }
   }
   if (__syncthreads_or(bad || (bad_block && threadIdx.x == 0)) && threadIdx.x == 0)
     atomicOr(J.status, (uint32_t)TMD_STATUS_CODED);
 }
 
-template <int W> struct Shape;
-template <> struct Shape<1> { static constexpr int kThreads = 256, kMinBlocks = 8; };
-template <> struct Shape<2> { static constexpr int kThreads = 512, kMinBlocks = 4; };
-template <> struct Shape<4> { static constexpr int kThreads = 512, kMinBlocks = 3; };
+__global__ void __launch_bounds__(kMaxThreads, 3) k_rans_decode(const __grid_constant__ Job J,
+                                                              uint32_t table_words) {
+  extern __shared__ __align__(16) uint32_t s_mem[];
+  int fi = 0;
+  while (fi + 1 < (int)J.nf && blockIdx.x >= J.f[fi + 1].block0) fi++;
+  const JobField& F = J.f[fi];
+  uint32_t* ring = s_mem + table_words;
+  if (F.width == 4) decode_block<4>(J, F, s_mem, ring);
+  else if (F.width == 2) decode_block<2>(J, F, s_mem, ring);
+  else decode_block<1>(J, F, s_mem, ring);
+}
 
-template <int W>
-cudaError_t launch_width(const uint8_t* coded, uint64_t bytes, const tmd_frame_arrays& dst,
-                         uint32_t* status, cudaStream_t st, uint32_t field_mask = ~0u) {
-  constexpr int kT = Shape<W>::kThreads, kB = Shape<W>::kMinBlocks;
+// Chunks (warps) of the streams in field_mask.
+uint32_t job_warps(const tmd_frame_arrays& d, uint32_t field_mask) {
+  uint32_t warps = 0;
+  for (int f = 0; f < kFields; f++)
+    if ((field_mask >> f) & 1u)
+      warps += std::max<uint32_t>(1, chunks_of(field_len(f, d.n_tracks, d.n_attached, d.n_unattached)));
+  return warps;
+}
+
+// Decodes the streams in field_mask.
+cudaError_t launch_streams(tmd_handle* h, const uint8_t* coded, uint64_t bytes,
+                           const tmd_frame_arrays& dst, uint32_t* status, cudaStream_t st,
+                           uint32_t field_mask = ~0u) {
   void* const ptr[kFields] = {dst.qpt,     dst.row,         dst.slice,        dst.pad,
                               dst.time,    dst.ncl,         dst.qtot_a,       dst.qmax_a,
                               dst.flags_a, dst.sigma_pad_a, dst.sigma_time_a, dst.row_diff,
@@ -428,26 +481,42 @@ cudaError_t launch_width(const uint8_t* coded, uint64_t bytes, const tmd_frame_a
   J.na = dst.n_attached;
   J.nu = dst.n_unattached;
   J.status = status;
-  uint32_t blocks = 0;
-  for (int f = 0; f < kFields; f++) {
-    if (kWidth[f] != (uint32_t)W || !((field_mask >> f) & 1u)) continue;
-    JobField& F = J.f[J.nf++];
-    F.dst = ptr[f];
-    F.n = field_len(f, J.nt, J.na, J.nu);
-    F.nch = chunks_of(F.n);
-    F.block0 = blocks;
-    F.index = (uint32_t)f;
-    // at least one block per stream, so that every directory entry is checked
-    blocks += std::max<uint32_t>(1, (F.nch + kT / 32 - 1) / (kT / 32));
-  }
+  // Blocks of 4, 8 or 16 chunks: a block shares its slot table among them, but
+  // the lane chains of a small frame run fastest spread over all the SMs.
+  const uint32_t warps = job_warps(dst, field_mask), sms = (uint32_t)h->sms;
+  const uint32_t threads = warps <= 4 * sms ? 128 : (warps <= 16 * sms ? 256 : kMaxThreads);
+  uint32_t blocks = 0, widest = 1;
+  for (uint32_t w = 4; w >= 1; w /= 2)
+    for (int f = 0; f < kFields; f++) {
+      if (kWidth[f] != w || !((field_mask >> f) & 1u)) continue;
+      JobField& F = J.f[J.nf++];
+      F.dst = ptr[f];
+      F.n = field_len(f, J.nt, J.na, J.nu);
+      F.nch = chunks_of(F.n);
+      F.block0 = blocks;
+      F.index = (uint32_t)f;
+      F.width = w;
+      widest = std::max(widest, w);
+      // at least one block per stream, so that every directory entry is checked
+      blocks += std::max<uint32_t>(1, (F.nch + threads / 32 - 1) / (threads / 32));
+    }
   if (J.nf == 0) return cudaSuccess;
-  const int smem = W * (int)kM * 4;
-  auto kern = k_rans_decode<W, kT, kB>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  kern<<<blocks, kT, smem, st>>>(J);
+  const uint32_t table_words = widest * kM;
+  const int smem =
+      4 * (int)(table_words + std::max<uint32_t>(threads * kRing, widest * kCumWords));
+  k_rans_decode<<<blocks, threads, smem, st>>>(J, table_words);
   return cudaGetLastError();
 }
+
+}  // namespace tmd_rans
+
+cudaError_t prepare_rans_decode() {
+  using namespace tmd_rans;
+  return cudaFuncSetAttribute(k_rans_decode, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              4 * (4 * (int)kM + kMaxThreads * kRing));
+}
+
+namespace tmd_rans {
 
 __global__ void k_status_or(uint32_t* dst, const uint32_t* src) { *dst |= *src; }
 
@@ -538,26 +607,7 @@ extern "C" int tmd_rans_decode(tmd_handle* h, const void* coded, uint64_t coded_
   if (rc != TMD_OK) return rc;
   const uint8_t* c = static_cast<const uint8_t*>(coded);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // the 4-byte streams (the fewest and longest lane streams) on the second
-  // stream beside the 2- and 1-byte streams, joined back at the end
-  const bool two = h->tune_rans_overlap && h->aux && h->fork && h->join;
-  if (two) {
-    rc = tmd_cuda_check(h, cudaEventRecord(h->fork, st), "cudaEventRecord");
-    if (rc == TMD_OK) rc = tmd_cuda_check(h, cudaStreamWaitEvent(h->aux, h->fork, 0), "cudaStreamWaitEvent");
-    if (rc != TMD_OK) return rc;
-  }
-  rc = tmd_cuda_check(h, launch_width<4>(c, coded_bytes, *dst, status, two ? h->aux : st),
-                      "k_rans_decode<4>");
-  if (rc != TMD_OK) return rc;
-  if (two) {
-    rc = tmd_cuda_check(h, cudaEventRecord(h->join, h->aux), "cudaEventRecord");
-    if (rc != TMD_OK) return rc;
-  }
-  rc = tmd_cuda_check(h, launch_width<2>(c, coded_bytes, *dst, status, st), "k_rans_decode<2>");
-  if (rc != TMD_OK) return rc;
-  rc = tmd_cuda_check(h, launch_width<1>(c, coded_bytes, *dst, status, st), "k_rans_decode<1>");
-  if (rc != TMD_OK || !two) return rc;
-  return tmd_cuda_check(h, cudaStreamWaitEvent(st, h->join, 0), "cudaStreamWaitEvent");
+  return tmd_cuda_check(h, launch_streams(h, c, coded_bytes, *dst, status, st), "k_rans_decode");
 }
 
 extern "C" int tmd_decode_coded_frame(tmd_handle* h, const void* coded, uint64_t coded_bytes,
@@ -626,30 +676,26 @@ extern "C" int tmd_decode_coded_frame(tmd_handle* h, const void* coded, uint64_t
                          (1u << 11) | (1u << 12) | (1u << 13) | (1u << 14) | (1u << 15);
   const uint32_t later = ((1u << kFields) - 1u) & ~first;
   // coded_overlap 1: the later streams start at once beside the first ones;
-  // 2: they start when the first ones are done (beside the track decoder only)
+  // 2: they start when the first ones are done (beside the track decoder only),
+  // unless the frame is so small (up to 8 chunks per SM) that both leave the
+  // GPU's issue slots mostly idle: then at once
   const bool two = h->tune_coded_overlap && h->aux && h->fork && h->coded_late;
-  if (two && h->tune_coded_overlap == 1) {
+  const bool at_once = two && (h->tune_coded_overlap == 1 ||
+                               job_warps(a, first | later) <= 8u * (uint32_t)h->sms);
+  if (at_once) {
     rc = tmd_cuda_check(h, cudaEventRecord(h->fork, st), "cudaEventRecord");
     if (rc == TMD_OK) rc = tmd_cuda_check(h, cudaStreamWaitEvent(h->aux, h->fork, 0), "cudaStreamWaitEvent");
     if (rc != TMD_OK) return rc;
   }
   const uint8_t* c = static_cast<const uint8_t*>(coded);
   cudaStream_t late_st = two ? h->aux : st;
-  rc = tmd_cuda_check(h, launch_width<4>(c, coded_bytes, a, cstatus, st, first), "k_rans_decode<4>");
-  if (rc == TMD_OK)
-    rc = tmd_cuda_check(h, launch_width<2>(c, coded_bytes, a, cstatus, st, first), "k_rans_decode<2>");
-  if (rc == TMD_OK)
-    rc = tmd_cuda_check(h, launch_width<1>(c, coded_bytes, a, cstatus, st, first), "k_rans_decode<1>");
-  if (rc == TMD_OK && two && h->tune_coded_overlap == 2) {
+  rc = tmd_cuda_check(h, launch_streams(h, c, coded_bytes, a, cstatus, st, first), "k_rans_decode");
+  if (rc == TMD_OK && two && !at_once) {
     rc = tmd_cuda_check(h, cudaEventRecord(h->fork, st), "cudaEventRecord");
     if (rc == TMD_OK) rc = tmd_cuda_check(h, cudaStreamWaitEvent(h->aux, h->fork, 0), "cudaStreamWaitEvent");
   }
   if (rc == TMD_OK)
-    rc = tmd_cuda_check(h, launch_width<4>(c, coded_bytes, a, cstatus, late_st, later), "k_rans_decode<4>");
-  if (rc == TMD_OK)
-    rc = tmd_cuda_check(h, launch_width<2>(c, coded_bytes, a, cstatus, late_st, later), "k_rans_decode<2>");
-  if (rc == TMD_OK)
-    rc = tmd_cuda_check(h, launch_width<1>(c, coded_bytes, a, cstatus, late_st, later), "k_rans_decode<1>");
+    rc = tmd_cuda_check(h, launch_streams(h, c, coded_bytes, a, cstatus, late_st, later), "k_rans_decode");
   if (rc == TMD_OK && two)
     rc = tmd_cuda_check(h, cudaEventRecord(h->coded_late, h->aux), "cudaEventRecord");
   if (rc != TMD_OK) return rc;
