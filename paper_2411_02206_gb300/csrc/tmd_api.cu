@@ -245,6 +245,7 @@ extern "C" int tmd_create(const tmd_config* cfg, tmd_handle** out) {
                            "event")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_count_rank(), "smem attribute")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_rans_decode(), "smem attribute")) != TMD_OK ||
+      (rc = tmd_cuda_check(h, prepare_global_xyz(&h->occ_xyz), "global transform")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_unatt_encode(&h->occ_ue), "unattached encoder")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_track_decode(0, &h->occ_decode_v[0]), "occupancy")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_track_decode(1, &h->occ_decode_v[1]), "occupancy")) != TMD_OK ||
@@ -260,6 +261,7 @@ extern "C" int tmd_create(const tmd_config* cfg, tmd_handle** out) {
   if (h->occ_unatt < 1) h->occ_unatt = 1;
   if (h->occ_encode < 1) h->occ_encode = 1;
   if (h->occ_ue < 1) h->occ_ue = 1;
+  if (h->occ_xyz < 1) h->occ_xyz = 1;
   *out = h;
   return TMD_OK;
 }

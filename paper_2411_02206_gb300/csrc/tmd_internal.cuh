@@ -152,6 +152,8 @@ __global__ void k_track_scan2(const FrameDev* frames, PlanDev plan);
 // (grid: ranking tiles of all frames).
 void launch_count_rank(uint32_t grid, cudaStream_t st, const FrameDev* frames, PlanDev plan);
 cudaError_t prepare_count_rank();
+// Shared-memory attribute of the tiled global transform; its resident blocks.
+cudaError_t prepare_global_xyz(int* blocks_per_sm);
 // Shared-memory attributes of the unattached encoder; resident blocks per SM
 // of its cooperative kernel.
 cudaError_t prepare_unatt_encode(int* blocks_per_sm);
