@@ -12,8 +12,8 @@
 // slot tables in shared memory (slot -> symbol, frequency, offset in one
 // u32), then every lane decodes its stream: per symbol one shared-memory
 // lookup, one multiply-add and, on renormalisation, the next 16-bit word from
-// a queue of the lane's own words that asynchronous copies keep kRing pairs
-// ahead (the words of a chunk are interleaved by lane, so a warp's copies of
+// a ring of the lane's own words that asynchronous copies keep kRing pairs
+// ahead, read ahead of need and without a branch (the words of a chunk are interleaved by lane, so a warp's copies of
 // pair j are one 128-byte line).  Values are written by the lane at positions
 // 32 k + l: a warp stores 32 consecutive values per step.  Streams of all
 // widths share a launch, the widest first: a lane's chain of 256 to 1024
@@ -249,8 +249,8 @@ void encode_stream(const void* vals, uint32_t n, unsigned threads, std::vector<u
 // ---------------------------------------------------------------------------
 // Device decoder
 // ---------------------------------------------------------------------------
-constexpr int kRing = 4;           // word pairs per lane in flight
-constexpr int kMaxThreads = 512;
+constexpr uint32_t kRing = 8;      // word pairs of a lane on chip
+constexpr int kMaxThreads = 768;
 constexpr int kCumWords = 257;     // cumulative frequencies of a plane
 
 struct JobField {
@@ -301,17 +301,55 @@ __device__ uint64_t check_entry(const Job& J, const JobField& F, uint32_t w) {
   return off;
 }
 
-// Copies one word pair to the lane's queue, or zeros if there is none.
-__device__ __forceinline__ void queue_pair(uint32_t* slot, const uint32_t* src, bool some) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(slot);
-  asm volatile(
-      "cp.async.ca.shared.global [%0], [%1], 4, %2;\n\t"
-      "cp.async.commit_group;" ::"r"(d), "l"(src), "r"(some ? 4 : 0) : "memory");
-}
-template <int N>
-__device__ __forceinline__ void queue_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
+// A lane's words: its pairs of the chunk, kRing of them in shared memory (one
+// word per lane and row of the ring: a warp's copies of one pair are one line,
+// its reads free of bank conflicts).  A step of at most four symbols takes at
+// most four words; it begins by queueing the pairs that the step before used
+// up and by taking its own four words into registers, which were queued two
+// steps earlier at the latest.
+struct Words {
+  uint32_t ring;         // shared-memory address of the lane's first pair
+  const uint32_t* next;  // pair number `queued`
+  uint32_t queued, have; // pairs queued, pairs there are
+  uint32_t used;         // words used
+  uint32_t w0, w1;       // the next four words, the first one lowest
+
+  // past the chunk's last pair nothing is copied: a stream that reads on is
+  // found by its count of words
+  __device__ __forceinline__ void queue() {
+    if (queued < have) {
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(ring + (queued % kRing) * 128),
+                   "l"(next) : "memory");
+      next += 32;
+    }
+    queued++;
+  }
+  __device__ __forceinline__ void start(uint32_t ring_, const uint32_t* first, uint32_t n) {
+    ring = ring_;
+    next = first;
+    have = n;
+    queued = used = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < kRing; i++) queue();
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+  }
+  __device__ __forceinline__ uint32_t pair(uint32_t row) const {
+    uint32_t w;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w) : "r"(ring + (row & (kRing * 128 - 128))));
+    return w;
+  }
+  __device__ __forceinline__ void begin_step() {
+    static_assert(kRing == 8, "see above");
+#pragma unroll
+    for (int i = 0; i < 2; i++)
+      if (queued < used / 2 + kRing) queue();
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 2;" ::: "memory");
+    const uint32_t row = used * 64, sh = used % 2 * 16;
+    const uint32_t a = pair(row), b = pair(row + 128), c = pair(row + 256);
+    w0 = __funnelshift_r(a, b, sh);
+    w1 = __funnelshift_r(b, c, sh);
+  }
+};
 
 // The chunks of one block, blockDim / 32 of them.  s_tab: W * 4096 slot
 // entries, symbol | (f - 1) << 8 | offset << 20; s_ring: kRing pairs per
@@ -400,18 +438,11 @@ __device__ __forceinline__ void decode_block(const Job& J, const JobField& F, ui
       if (w1 < w0 || ((w1 - w0) & 31u) || w1 > slots) bad = true;
       else maxp = (w1 - w0) >> 5;
       const uint32_t* P = reinterpret_cast<const uint32_t*>(sec + a_words) + w0 + lane;
-      uint32_t* ring = s_ring + warp * (32 * kRing) + lane;
-#pragma unroll
-      for (uint32_t i = 0; i < (uint32_t)kRing; i++) {
-        queue_pair(ring + 32 * i, P, i < maxp);
-        P += 32;
-      }
+      Words words;
+      words.start((uint32_t)__cvta_generic_to_shared(s_ring + warp * (32 * kRing) + lane), P, maxp);
       uint32_t x = st[32ull * chunk + lane];
-      queue_wait<kRing - 1>();
-      uint32_t cur = ring[0];  // the next word in its low half
-      uint32_t j = 0;          // pair held in cur
-      bool half = false;       // its first word is used
-      for (uint32_t k = 0; k < nk; k++) {
+      uint32_t low = 0xFFFFFFFFu;  // smallest state after a symbol
+      auto value = [&]() {
         uint32_t v = 0;
 #pragma unroll
         for (int p = 0; p < W; p++) {
@@ -420,30 +451,36 @@ __device__ __forceinline__ void decode_block(const Job& J, const JobField& F, ui
           x = ((e >> 8) & (kM - 1)) * xs + xs + (e >> 20);
           v = __byte_perm(v, e, p == 0 ? 0x3214 : p == 1 ? 0x3240 : p == 2 ? 0x3410 : 0x4210);
           if (x < kLower) {
-            x = __byte_perm(cur, x, 0x5410);
-            if (x < kLower) bad = true;
-            cur >>= 16;
-            if (half) {
-              queue_pair(ring + 32 * (j % kRing), P, j + kRing < maxp);
-              P += 32;
-              j++;
-              queue_wait<kRing - 1>();
-              cur = ring[32 * (j % kRing)];
-            }
-            half = !half;
+            x = __byte_perm(words.w0, x, 0x5410);
+            words.w0 = __byte_perm(words.w0, words.w1, 0x5432);
+            words.w1 >>= 16;
+            words.used++;
           }
+          low = min(low, x);
         }
-        out[32ull * k] = (T)v;
+        return (T)v;
+      };
+      constexpr uint32_t V = 4 / W;  // values per step of four symbols
+      uint32_t k = 0;
+      for (; k + V <= nk; k += V) {
+        words.begin_step();
+#pragma unroll
+        for (uint32_t u = 0; u < V; u++) out[32ull * (k + u)] = value();
       }
-      // every word came from the chunk, and the encoder's start state is left
-      if (2 * j + (half ? 1u : 0u) > 2 * maxp || x != kLower) bad = true;
+      for (; k < nk; k++) {
+        words.begin_step();
+        out[32ull * k] = value();
+      }
+      // every word came from the chunk, no state was left below the interval,
+      // and the encoder's start state remains
+      if (words.used > 2 * maxp || low < kLower || x != kLower) bad = true;
     }
   }
   if (__syncthreads_or(bad || (bad_block && threadIdx.x == 0)) && threadIdx.x == 0)
     atomicOr(J.status, (uint32_t)TMD_STATUS_CODED);
 }
 
-__global__ void __launch_bounds__(kMaxThreads, 3) k_rans_decode(const __grid_constant__ Job J,
+__global__ void __launch_bounds__(kMaxThreads, 2) k_rans_decode(const __grid_constant__ Job J,
                                                               uint32_t table_words) {
   extern __shared__ __align__(16) uint32_t s_mem[];
   int fi = 0;
@@ -481,10 +518,10 @@ cudaError_t launch_streams(tmd_handle* h, const uint8_t* coded, uint64_t bytes,
   J.na = dst.n_attached;
   J.nu = dst.n_unattached;
   J.status = status;
-  // Blocks of 4, 8 or 16 chunks: a block shares its slot table among them, but
+  // Blocks of 4, 8 or 24 chunks: a block shares its slot table among them, but
   // the lane chains of a small frame run fastest spread over all the SMs.
   const uint32_t warps = job_warps(dst, field_mask), sms = (uint32_t)h->sms;
-  const uint32_t threads = warps <= 4 * sms ? 128 : (warps <= 16 * sms ? 256 : kMaxThreads);
+  const uint32_t threads = warps <= 4 * sms ? 128 : (warps <= 12 * sms ? 256 : kMaxThreads);
   uint32_t blocks = 0, widest = 1;
   for (uint32_t w = 4; w >= 1; w /= 2)
     for (int f = 0; f < kFields; f++) {
