@@ -6,9 +6,11 @@
 //
 //   k_put_record: frame descriptors and prefix tables, scratch cleared
 //   k_zero_status -> k_track_scan1 -> k_frame_scan -> k_track_scan2   track prep
+//     (calls of small frames: k_track_prep)
 //   k_track_decode: coordinates and (sector,row) keys                  track decode
 //   k_count_rank: per-tile counts and stable ranks                     per-row counts
 //   k_group_sum -> k_row_offsets -> k_tile_base                        row offsets
+//     (frames of one group of tiles: without k_group_sum)
 //   k_att_scatter: native records of the attached clusters             placement
 //   k_unatt_decode                                                     unattached clusters
 #include <cstdio>
@@ -284,7 +286,7 @@ extern "C" const char* tmd_last_error_string(const tmd_handle* h) {
 static const char* kKernelNames[kKNum] = {
     "k_put_record", "k_zero_status", "k_track_scan1", "k_frame_scan", "k_track_scan2",
     "k_track_decode", "k_count_rank", "k_group_sum", "k_row_offsets", "k_tile_base",
-    "k_att_scatter", "k_unatt_decode", "k_track_encode"};
+    "k_att_scatter", "k_unatt_decode", "k_track_encode", "k_track_prep"};
 
 cudaEvent_t TmdProfile::get() {
   if (pool.empty()) {
@@ -441,6 +443,9 @@ int tmd_enqueue(tmd_handle* h, uint32_t nf, const tmd_frame_in* in, const tmd_fr
   EncDev* ed = reinterpret_cast<EncDev*>(host + R.enc);
   pre_tblk[0] = pre_tile[0] = pre_grp[0] = pre_warp[0] = pre_chunk[0] = pre_kt[0] = 0;
   uint32_t* zero_bins = reinterpret_cast<uint32_t*>(zb + 256);
+  uint64_t all_tracks = 0;
+  for (uint32_t f = 0; f < nf; f++) all_tracks += encode ? tin[f].n_tracks : in[f].n_tracks;
+  const uint32_t lanes = task_lanes(all_tracks, (uint32_t)h->sms);
   for (uint32_t f = 0; f < nf; f++) {
     FrameDev& F = fd[f];
     memset(&F, 0, sizeof F);
@@ -493,9 +498,9 @@ int tmd_enqueue(tmd_handle* h, uint32_t nf, const tmd_frame_in* in, const tmd_fr
     pre_tblk[f + 1] = pre_tblk[f] + l.n_tblocks;
     pre_tile[f + 1] = pre_tile[f] + l.n_tiles;
     pre_grp[f + 1] = pre_grp[f] + l.n_groups * kBinBlocks;
-    pre_warp[f + 1] = pre_warp[f] + ceil_div(F.n_tracks, 32);  // encoder warp tasks
+    pre_warp[f + 1] = pre_warp[f] + ceil_div(F.n_tracks, lanes);  // encoder warp tasks
     pre_chunk[f + 1] = pre_chunk[f] + l.n_chunks;
-    pre_kt[f + 1] = pre_kt[f] + ceil_div(F.n_tracks, 32);
+    pre_kt[f + 1] = pre_kt[f] + ceil_div(F.n_tracks, lanes);
   }
   PlanDev P;
   const uint32_t* dpre = reinterpret_cast<const uint32_t*>(dev + R.pre);
@@ -506,6 +511,7 @@ int tmd_enqueue(tmd_handle* h, uint32_t nf, const tmd_frame_in* in, const tmd_fr
   P.pre_warp = dpre + 3 * (nf + 1);
   P.pre_chunk = dpre + 4 * (nf + 1);
   P.pre_kt = dpre + 5 * (nf + 1);
+  P.lanes = lanes;
   P.counters = reinterpret_cast<uint32_t*>(zb);
   const FrameDev* dframes = reinterpret_cast<const FrameDev*>(dev + R.frames);
   const EncDev* denc = reinterpret_cast<const EncDev*>(dev + R.enc);
@@ -535,9 +541,19 @@ int tmd_enqueue(tmd_handle* h, uint32_t nf, const tmd_frame_in* in, const tmd_fr
   if (!zs) timed(kKZeroStatus, [&] { k_zero_status<<<1, 256, 0, st>>>(dframes, nf); });
   const uint32_t n_tblk = pre_tblk[nf], n_tile = pre_tile[nf], n_grp = pre_grp[nf];
   const uint32_t n_warp = pre_warp[nf], n_chunk = pre_chunk[nf];
-  if (n_tblk) timed(kKTrackScan1, [&] { k_track_scan1<<<n_tblk, 256, 0, st>>>(dframes, P); });
-  timed(kKFrameScan, [&] { k_frame_scan<<<nf, 1024, 0, st>>>(dframes, P); });
-  if (n_tblk) timed(kKTrackScan2, [&] { k_track_scan2<<<n_tblk, 256, 0, st>>>(dframes, P); });
+  // calls of small frames only: one kernel for the track preparation
+  uint32_t most_tracks = 0, most_tiles = 0;
+  for (uint32_t f = 0; f < nf; f++) {
+    most_tracks = std::max(most_tracks, fd[f].n_tracks);
+    most_tiles = std::max(most_tiles, fd[f].n_tiles);
+  }
+  if (most_tracks <= (uint32_t)kPrepTracks) {
+    timed(kKTrackPrep, [&] { k_track_prep<<<dim3(nf, 2), 1024, 0, st>>>(dframes); });
+  } else {
+    if (n_tblk) timed(kKTrackScan1, [&] { k_track_scan1<<<n_tblk, 256, 0, st>>>(dframes, P); });
+    timed(kKFrameScan, [&] { k_frame_scan<<<nf, 1024, 0, st>>>(dframes, P); });
+    if (n_tblk) timed(kKTrackScan2, [&] { k_track_scan2<<<n_tblk, 256, 0, st>>>(dframes, P); });
+  }
   if (trace) {
     if (trace->n)
       k_track_trace<<<(trace->n + 127) / 128, 128, 0, st>>>(dframes, trace->ids, trace->n,
@@ -580,8 +596,11 @@ int tmd_enqueue(tmd_handle* h, uint32_t nf, const tmd_frame_in* in, const tmd_fr
           (uint32_t)(h->sms * bps), (n_kt + per_block - 1) / per_block));
       timed(kKTrackDecode, [&] { launch_track_decode(var, grid, st, dframes, P, n_kt); });
     }
-    if (n_tile) timed(kKCountRank, [&] { launch_count_rank(n_tile, st, dframes, P); });
-    if (n_grp) timed(kKGroupSum, [&] { k_group_sum<<<n_grp, kBinBlk, 0, st>>>(dframes, P); });
+    const bool groups = most_tiles > (uint32_t)kGroup;
+    if (n_tile)
+      timed(kKCountRank, [&] { launch_count_rank(n_tile, !groups, (uint32_t)h->sms, st, dframes, P); });
+    if (groups)
+      timed(kKGroupSum, [&] { k_group_sum<<<n_grp, kBinBlk, 0, st>>>(dframes, P); });
     timed(kKRowOffsets, [&] { k_row_offsets<<<nf, 1024, 0, st>>>(dframes, P); });
     auto unatt = [&](cudaStream_t s_) {
       if (!n_chunk) return;

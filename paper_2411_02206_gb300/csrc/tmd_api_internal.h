@@ -18,6 +18,7 @@ struct TmdServer;  // serving state (tmd_serve.cu)
 enum TmdKernel {
   kKPutRecord, kKZeroStatus, kKTrackScan1, kKFrameScan, kKTrackScan2, kKTrackDecode,
   kKCountRank, kKGroupSum, kKRowOffsets, kKTileBase, kKAttScatter, kKUnattDecode, kKTrackEncode,
+  kKTrackPrep,
   kKNum
 };
 

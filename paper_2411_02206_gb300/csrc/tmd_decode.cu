@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kDecodeThreads, MINB)
   fill_row_geo(&geo_s);
   __syncthreads();
   const RowGeo* geo = &geo_s;
-  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t lane = threadIdx.x & 31, lanes = plan.lanes;
   const uint32_t sq = lane % R, sg = lane / R;
   AsyncStage<R>& S = reinterpret_cast<AsyncStage<R>*>(s_stage)[threadIdx.x >> 5];
   for (;;) {
@@ -163,7 +163,8 @@ __global__ void __launch_bounds__(kDecodeThreads, MINB)
     const uint32_t f = find_frame(plan.pre_kt, plan.n_frames, task);
     const FrameDev& F = frames[f];
     if (*F.status & kStCount) continue;
-    const uint32_t idx = (task - plan.pre_kt[f]) * 32u + lane;
+    const uint32_t idx =
+        lane < lanes ? (task - plan.pre_kt[f]) * lanes + lane : 0xFFFFFFFFu;
     const uint8_t* __restrict__ rd_s = F.row_diff;
     const uint8_t* __restrict__ sld_s = F.sld;
     const uint16_t* __restrict__ pr_s = F.pad_res;
@@ -237,10 +238,12 @@ __global__ void __launch_bounds__(kDecodeThreads, MINB)
       }
       // rounds in which every lane has all R steps left run without the
       // per-step bound test (the common case for the long tracks decoded first)
-      const bool full = __all_sync(kFull, rem >= (uint32_t)R);
+      const bool full = __all_sync(kFull, rem >= (uint32_t)R || lane >= lanes);
       if (full) {
+        if (lane < lanes) {
 #pragma unroll 4
-        for (uint32_t q = q0; q < (uint32_t)R; q++) step(q);
+          for (uint32_t q = q0; q < (uint32_t)R; q++) step(q);
+        }
       } else {
 #pragma unroll 1
         for (uint32_t q = q0; q < (uint32_t)R; q++)
@@ -251,6 +254,7 @@ __global__ void __launch_bounds__(kDecodeThreads, MINB)
       const uint32_t* bb = ((r & 1) ? S.buf[1] : S.buf[0]) + Lay::kTr + (int)sq - 1;
 #pragma unroll
       for (int i0 = 0; i0 < 32; i0 += G) {
+        if (i0 >= (int)lanes) break;
         const uint32_t i = i0 + sg;
         const uint32_t ji = __shfl_sync(kFull, j0, i);
         // length and time offset of track i; in a full round every track has step k
@@ -380,7 +384,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 3)
   fill_row_geo(&geo);
   __syncthreads();
   EncStage& S = reinterpret_cast<EncStage*>(s_stage)[threadIdx.x >> 5];
-  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t lane = threadIdx.x & 31, lanes = plan.lanes;
   const uint32_t sq = lane % R, sg = lane / R;
   for (;;) {
     const uint32_t task = next_task(&plan.counters[0]);
@@ -389,7 +393,8 @@ __global__ void __launch_bounds__(kDecodeThreads, 3)
     const FrameDev& F = frames[f];
     const EncDev& D = enc[f];
     if (*F.status & kStCount) continue;
-    const uint32_t idx = (task - plan.pre_warp[f]) * 32u + lane;
+    const uint32_t idx =
+        lane < lanes ? (task - plan.pre_warp[f]) * lanes + lane : 0xFFFFFFFFu;
     // in registers: stores to the output bytes may alias the descriptor
     const Truth E{D.row, D.sector, D.leg, D.pad, D.time};
     uint8_t* __restrict__ rd_o = D.o_row_diff;
@@ -468,10 +473,12 @@ __global__ void __launch_bounds__(kDecodeThreads, 3)
         time_b[q] = timeq - ptime;
         update(G, s, padq, timeq);
       };
-      const bool full = __all_sync(kFull, rem >= (uint32_t)R);
+      const bool full = __all_sync(kFull, rem >= (uint32_t)R || lane >= lanes);
       if (full) {
+        if (lane < lanes) {
 #pragma unroll 4
-        for (uint32_t q = q0; q < (uint32_t)R; q++) step(q);
+          for (uint32_t q = q0; q < (uint32_t)R; q++) step(q);
+        }
       } else {
 #pragma unroll 1
         for (uint32_t q = q0; q < (uint32_t)R; q++)
@@ -480,8 +487,9 @@ __global__ void __launch_bounds__(kDecodeThreads, 3)
       __syncwarp();
       const uint32_t k = k0 + sq;
       const uint32_t* bb = (r & 1) ? S.buf[1] : S.buf[0];
-#pragma unroll 8
+#pragma unroll
       for (int i0 = 0; i0 < 32; i0 += 32 / R) {
+        if (i0 >= (int)lanes) break;
         const uint32_t i = i0 + sg;
         const uint32_t di = __shfl_sync(kFull, dm1, i) + k;
         const uint32_t no = __shfl_sync(kFull, n | ((uint32_t)o_time << 16), i);

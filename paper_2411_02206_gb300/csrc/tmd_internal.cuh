@@ -11,8 +11,6 @@ namespace tmd {
 // Work decomposition (fixed by the decoder, independent of the GPU model).
 constexpr int kTrackBlk = 2048;          // tracks per block of the track scan
 constexpr int kTile = 32768;             // attached clusters per ranking tile
-constexpr int kTileWarps = 8;            // warps per ranking tile
-constexpr int kTileSub = kTile / kTileWarps;  // clusters per warp of a tile
 constexpr int kGroup = 32;               // tiles per group of the tile scan
 constexpr int kBinBlk = 256;             // bins per block of the tile scan
 constexpr int kBinBlocks = (kNBin + kBinBlk - 1) / kBinBlk;
@@ -103,11 +101,26 @@ struct PlanDev {
   const uint32_t* pre_tblk;   // track-scan blocks
   const uint32_t* pre_tile;   // ranking tiles
   const uint32_t* pre_grp;    // tile-group blocks (n_groups * kBinBlocks)
-  const uint32_t* pre_warp;   // encoder: warp tasks of 32 tracks
+  const uint32_t* pre_warp;   // encoder: warp tasks
   const uint32_t* pre_chunk;  // unattached chunks
-  const uint32_t* pre_kt;     // decoder: warp tasks of 32 tracks
+  const uint32_t* pre_kt;     // decoder: warp tasks
+  uint32_t lanes;             // tracks per warp task (task_lanes)
   uint32_t* counters;         // [0] decode/encode task, [1] unattached ticket (zeroed)
 };
+
+// Tracks per warp task of the track decoder and encoder, one lane each.  A call
+// whose tracks fill all resident warps takes 32.  A smaller call is as long as
+// its longest track's chain of steps, and a step is the longer the more lanes
+// share it (a lane's sector change holds up the others; every track of the
+// warp is written out): it takes fewer lanes as long as its tasks are resident
+// together.  2000 tracks: 61 us at 32 lanes,
+// 41 us at 4; 11 111 tracks: 62 us at 32, 51 us at 8.
+inline uint32_t task_lanes(uint64_t n_tracks, uint32_t sms) {
+  const uint64_t warps = 12ull * sms;  // 3 blocks of 4 warps per SM
+  for (uint32_t l = 4; l < 32; l *= 2)
+    if (n_tracks <= l * warps) return l;
+  return 32;
+}
 
 // Largest f with pre[f] <= item (pre has n+1 entries, pre[0] = 0).
 __device__ __forceinline__ uint32_t find_frame(const uint32_t* pre, uint32_t n, uint32_t item) {
@@ -148,9 +161,16 @@ __global__ void k_zero_status(const FrameDev* frames, uint32_t n_frames);
 __global__ void k_track_scan1(const FrameDev* frames, PlanDev plan);
 __global__ void k_frame_scan(const FrameDev* frames, PlanDev plan);
 __global__ void k_track_scan2(const FrameDev* frames, PlanDev plan);
+// The same for frames of at most kPrepTracks tracks (grid: frames x 2).
+constexpr int kPrepTracks = 16384;
+__global__ void k_track_prep(const FrameDev* frames);
 // Tile histograms and stable ranks of the attached clusters from their keys
 // (grid: ranking tiles of all frames).
-void launch_count_rank(uint32_t grid, cudaStream_t st, const FrameDev* frames, PlanDev plan);
+// With sum, the tiles' counts are added into the bins' attached counts here:
+// calls whose frames are of one group of tiles each need no k_group_sum (4.5 us
+// and a launch; with many tiles the adds slow the ranking more than that).
+void launch_count_rank(uint32_t n_tiles, bool sum, uint32_t sms, cudaStream_t st,
+                       const FrameDev* frames, PlanDev plan);
 cudaError_t prepare_count_rank();
 // Shared-memory attribute of the tiled global transform; its resident blocks.
 cudaError_t prepare_global_xyz(int* blocks_per_sm);
@@ -162,8 +182,8 @@ __global__ void k_row_offsets(const FrameDev* frames, PlanDev plan);
 __global__ void k_tile_base(const FrameDev* frames, PlanDev plan);
 // The track decoder is instantiated in variants of its staging (a tuning
 // parameter, every instance computes identical results); host code launches
-// it through these two functions.  Its warps take tasks of 32 tracks (pre_kt
-// of the plan) from counters[0] and write the key, pad code and time code of
+// it through these two functions.  Its warps take tasks of plan.lanes tracks
+// (pre_kt of the plan) from counters[0] and write the key, pad code and time code of
 // every attached cluster.
 void launch_track_decode(int variant, uint32_t grid, cudaStream_t st, const FrameDev* frames,
                          PlanDev plan, uint32_t n_tasks);
@@ -186,6 +206,5 @@ __global__ void k_track_trace(const FrameDev* frames, const uint32_t* ids, uint3
 
 constexpr int kRankTags = 2048;  // per-warp duplicate-test slots of the ranking (bytes)
 constexpr int kRankGroup = 2;    // ranking steps tested for distinct keys at once
-constexpr int kCountRankSmem = kTileWarps * kNBin * 2 + kTileWarps * kRankTags;
 
 }  // namespace tmd

@@ -150,7 +150,8 @@ extern "C" int tmd_decode_frame_noalloc(const tmd_frame_in* in, const tmd_frame_
   F.unatt_start = reinterpret_cast<uint32_t*>(pb + L.unatt_start);
   F.blk_sum = reinterpret_cast<uint32_t*>(pb + L.blk_sum);
   const uint32_t n_tblk = L.n_tblocks, n_tile = L.n_tiles, n_grp = L.n_groups * kBinBlocks;
-  const uint32_t n_kt = (in->n_tracks + 31) / 32;  // decoder warp tasks
+  const uint32_t lanes = task_lanes(in->n_tracks, (uint32_t)S->sms);
+  const uint32_t n_kt = (in->n_tracks + lanes - 1) / lanes;  // decoder warp tasks
   const uint32_t n_warp = n_kt;
   const uint32_t n_chunk = L.n_chunks;
   FrameDev* dframe = reinterpret_cast<FrameDev*>(rec);
@@ -163,6 +164,7 @@ extern "C" int tmd_decode_frame_noalloc(const tmd_frame_in* in, const tmd_frame_
   P.pre_warp = dpre + 6;
   P.pre_chunk = dpre + 8;
   P.pre_kt = dpre + 10;
+  P.lanes = lanes;
   P.counters = reinterpret_cast<uint32_t*>(zb);
   k_noalloc_record<<<1, 32, 0, st>>>(F, n_tblk, n_tile, n_grp, n_warp, n_chunk, n_kt, dframe,
                                      dpre);
@@ -179,8 +181,8 @@ extern "C" int tmd_decode_frame_noalloc(const tmd_frame_in* in, const tmd_frame_
     const uint32_t want = (n_kt + kDecodeThreads / 32 - 1) / (kDecodeThreads / 32);
     launch_track_decode(0, want < cap ? want : cap, st, dframe, P, n_kt);
   }
-  if (n_tile) launch_count_rank(n_tile, st, dframe, P);
-  if (n_grp) k_group_sum<<<n_grp, kBinBlk, 0, st>>>(dframe, P);
+  if (n_tile) launch_count_rank(n_tile, L.n_groups <= 1, (uint32_t)S->sms, st, dframe, P);
+  if (L.n_groups > 1) k_group_sum<<<n_grp, kBinBlk, 0, st>>>(dframe, P);
   k_row_offsets<<<1, 1024, 0, st>>>(dframe, P);
   if (n_grp) k_tile_base<<<n_grp, kBinBlk, 0, st>>>(dframe, P);
   if (n_tile) launch_att_scatter(1, n_tile, st, dframe, P);

@@ -33,8 +33,17 @@
 
 namespace tmd {
 
-__global__ void __launch_bounds__(256, 2) k_count_rank(const FrameDev* frames, PlanDev plan) {
-  // [kTileWarps][kNBin/2] packed u16 counts, then [kTileWarps][kRankTags] byte slots
+template <int W>
+constexpr int kRankSmem = W * (kNBin * 2 + kRankTags);
+
+// W warps per tile: 8 with two blocks per SM, or 16 when the call has no more
+// tiles than SMs (a warp's clusters are one serial chain: 20 us with 8 warps
+// for a frame of 190 k clusters, 18 us with 16).
+template <int W>
+__global__ void __launch_bounds__(32 * W, 16 / W) k_count_rank(const FrameDev* frames, PlanDev plan,
+                                                            bool sum) {
+  // [W][kNBin/2] packed u16 counts, then [W][kRankTags] byte slots
+  constexpr int kTileWarps = W, kTileSub = kTile / W;
   extern __shared__ uint32_t s_mem[];
   const uint32_t f = find_frame(plan.pre_tile, plan.n_frames, blockIdx.x);
   const FrameDev& F = frames[f];
@@ -91,6 +100,7 @@ __global__ void __launch_bounds__(256, 2) k_count_rank(const FrameDev* frames, P
       run += c;
     }
     tile_hist[(size_t)tile * kNBin + b] = (uint16_t)run;
+    if (sum && run) atomicAdd(&F.att_count[b], run);
   }
   __syncthreads();
   // pass 2: stable ranks in stream order; the keys of the next 8 steps are
@@ -181,13 +191,21 @@ __global__ void __launch_bounds__(256, 2) k_count_rank(const FrameDev* frames, P
   }
 }
 
-void launch_count_rank(uint32_t grid, cudaStream_t st, const FrameDev* frames, PlanDev plan) {
-  k_count_rank<<<grid, 256, kCountRankSmem, st>>>(frames, plan);
+void launch_count_rank(uint32_t n_tiles, bool sum, uint32_t sms, cudaStream_t st,
+                       const FrameDev* frames, PlanDev plan) {
+  if (n_tiles <= sms)
+    k_count_rank<16><<<n_tiles, 512, kRankSmem<16>, st>>>(frames, plan, sum);
+  else
+    k_count_rank<8><<<n_tiles, 256, kRankSmem<8>, st>>>(frames, plan, sum);
 }
 
 cudaError_t prepare_count_rank() {
-  return cudaFuncSetAttribute(k_count_rank, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              kCountRankSmem);
+  cudaError_t e = cudaFuncSetAttribute(k_count_rank<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       kRankSmem<8>);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_count_rank<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kRankSmem<16>);
+  return e;
 }
 
 }  // namespace tmd

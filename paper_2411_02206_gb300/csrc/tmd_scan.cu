@@ -151,6 +151,34 @@ __global__ void __launch_bounds__(256) k_track_scan1(const FrameDev* frames, Pla
     if (hist[i]) atomicAdd(&F.len_cursor[i], hist[i]);
 }
 
+// Starts of the unattached bins (six consecutive bins per thread, one scan),
+// their total checked, and the attached counts per bin cleared; one block of
+// 1024 threads.
+__device__ __forceinline__ void unatt_bins(const FrameDev& F) {
+  constexpr int Q = (kNBin + 1023) / 1024;
+  const uint32_t tid = threadIdx.x, b0 = tid * Q;
+  uint32_t v[Q], sum = 0, tot;
+#pragma unroll
+  for (int q = 0; q < Q; q++) {
+    v[q] = b0 + q < (uint32_t)kNBin ? F.n_unatt_bin[b0 + q] : 0u;
+    sum += v[q];
+  }
+  uint32_t run = block_excl_scan<1024>(sum, tot);
+#pragma unroll
+  for (int q = 0; q < Q; q++) {
+    if (b0 + q < (uint32_t)kNBin) F.unatt_start[b0 + q] = run;
+    run += v[q];
+  }
+  if (tid == 0) {
+    F.unatt_start[kNBin] = tot;
+    if (tot != F.n_unatt) atomicOr(F.status, kStCount);
+  }
+  // attached counts per bin: summed into by k_count_rank or k_group_sum (an
+  // encoding call has none)
+  if (F.att_count)
+    for (uint32_t b = tid; b < (uint32_t)kNBin; b += 1024) F.att_count[b] = 0u;
+}
+
 // Per frame: offsets of the track blocks, decode-order bucket offsets (longest
 // first), unattached bin starts, count checks.
 __global__ void __launch_bounds__(1024) k_frame_scan(const FrameDev* frames, PlanDev plan) {
@@ -172,32 +200,7 @@ __global__ void __launch_bounds__(1024) k_frame_scan(const FrameDev* frames, Pla
     const uint32_t e = block_excl_scan<1024>(v, tot);
     F.len_cursor[b] = e;
   }
-  {
-    // unattached bin starts: kBinPerThread consecutive bins per thread, one scan
-    constexpr int Q = (kNBin + 1023) / 1024;
-    uint32_t v[Q], sum = 0;
-    const uint32_t b0 = tid * Q;
-#pragma unroll
-    for (int q = 0; q < Q; q++) {
-      v[q] = b0 + q < (uint32_t)kNBin ? F.n_unatt_bin[b0 + q] : 0u;
-      sum += v[q];
-    }
-    uint32_t run = block_excl_scan<1024>(sum, tot);
-#pragma unroll
-    for (int q = 0; q < Q; q++) {
-      if (b0 + q < (uint32_t)kNBin) F.unatt_start[b0 + q] = run;
-      run += v[q];
-    }
-    carry = tot;
-  }
-  if (tid == 0) {
-    F.unatt_start[kNBin] = (uint32_t)carry;
-    if (carry != F.n_unatt) atomicOr(F.status, kStCount);
-  }
-  // attached counts per bin: summed into by k_group_sum (an encoding call
-  // has none)
-  if (F.att_count)
-    for (uint32_t b = tid; b < (uint32_t)kNBin; b += 1024) F.att_count[b] = 0u;
+  unatt_bins(F);
 }
 
 // trackStart and decode order.  A block first counts its tracks per length
@@ -246,8 +249,62 @@ __global__ void __launch_bounds__(256) k_track_scan2(const FrameDev* frames, Pla
   }
 }
 
+// The whole track preparation of frames of at most kPrepTracks tracks in one
+// launch, two blocks per frame (tracks; unattached bins): a call of small
+// frames is a chain of latencies, and the three kernels above take 25 us
+// for 2000 tracks where this one takes 8 us.
+__global__ void __launch_bounds__(1024) k_track_prep(const FrameDev* frames) {
+  __shared__ uint32_t s_cur[kLenBuckets];
+  const FrameDev& F = frames[blockIdx.x];
+  if (blockIdx.y == 1) {
+    unatt_bins(F);
+    return;
+  }
+  constexpr int E = kPrepTracks / 1024;
+  const uint32_t tid = threadIdx.x, nt = F.n_tracks;
+  const uint32_t per = (nt + 1023) / 1024;  // consecutive tracks per thread, at most E
+  const uint16_t* __restrict__ ncl = F.ncl;
+  static_assert(kLenBuckets == 1024, "one bucket per thread");
+  s_cur[tid] = 0u;
+  __syncthreads();
+  uint32_t n[E], sum = 0, tot;
+  bool zero = false;
+#pragma unroll
+  for (int k = 0; k < E; k++) {
+    const uint32_t t = tid * per + k;
+    const bool in = (uint32_t)k < per && t < nt;
+    n[k] = in ? (uint32_t)ncl[t] : 0u;
+    sum += n[k];
+    zero |= in && n[k] == 0;
+    if (in) atomicAdd(&s_cur[min(n[k], (uint32_t)kLenBuckets - 1)], 1u);
+  }
+  uint32_t start = block_excl_scan<1024>(sum, tot);  // at most 2^14 * 65535: no overflow
+  if (__syncthreads_or(zero) || tot != F.n_att) {
+    if (tid == 0) atomicOr(F.status, kStCount);
+    return;
+  }
+  // buckets in descending length
+  const uint32_t b = kLenBuckets - 1 - tid, v = s_cur[b];
+  const uint32_t e = block_excl_scan<1024>(v, tot);
+  s_cur[b] = e;
+  __syncthreads();
+  uint32_t* __restrict__ track_start = F.track_start;
+  uint32_t* __restrict__ order = F.order;
+#pragma unroll
+  for (int k = 0; k < E; k++) {
+    const uint32_t t = tid * per + k;
+    if ((uint32_t)k < per && t < nt) {
+      track_start[t] = start;
+      order[atomicAdd(&s_cur[min(n[k], (uint32_t)kLenBuckets - 1)], 1u)] = t;
+      start += n[k];
+      if (t == nt - 1) track_start[nt] = start;
+    }
+  }
+}
+
 // Sum of the tile histograms over groups of kGroup tiles, per bin; the group
 // sums are also added into the bin's attached count (cleared by k_frame_scan).
+// Calls with a frame of several groups; see launch_count_rank.
 __global__ void __launch_bounds__(kBinBlk) k_group_sum(const FrameDev* frames, PlanDev plan) {
   const uint32_t f = find_frame(plan.pre_grp, plan.n_frames, blockIdx.x);
   const FrameDev& F = frames[f];
@@ -288,7 +345,7 @@ __device__ __forceinline__ void row_start_scan(const FrameDev& F) {
   if (threadIdx.x == 0) F.row_start[kNBin] = tot;
 }
 
-// Per frame: rowStart (the attached counts were summed by k_group_sum).
+// Per frame: rowStart (the attached counts are there).
 __global__ void __launch_bounds__(1024) k_row_offsets(const FrameDev* frames, PlanDev plan) {
   const FrameDev& F = frames[blockIdx.x];
   if (*F.status & kStCount) return;
