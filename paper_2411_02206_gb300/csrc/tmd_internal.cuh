@@ -113,8 +113,8 @@ struct PlanDev {
 // its longest track's chain of steps, and a step is the longer the more lanes
 // share it (a lane's sector change holds up the others; every track of the
 // warp is written out): it takes fewer lanes as long as its tasks are resident
-// together.  2000 tracks: 61 us at 32 lanes,
-// 41 us at 4; 11 111 tracks: 62 us at 32, 51 us at 8.
+// together.  2000 tracks: 61 us at 32 lanes, 41 us at 4; 11 111 tracks: 62 us at
+// 32, 51 us at 8.
 inline uint32_t task_lanes(uint64_t n_tracks, uint32_t sms) {
   const uint64_t warps = 12ull * sms;  // 3 blocks of 4 warps per SM
   for (uint32_t l = 4; l < 32; l *= 2)

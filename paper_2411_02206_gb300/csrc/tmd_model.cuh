@@ -102,13 +102,22 @@ __device__ __forceinline__ void fill_row_geo(RowGeo* g) {
   }
 }
 
-// Quantiser: clamp to [lo, hi] (NaN to lo), then floor(v + 0.5).  fmaxf
-// returns its non-NaN operand, so NaN clamps to lo; v + 0.5 then lies in
-// [0.5, hi + 0.5] with lo = 0, where the round-down conversion to unsigned
-// equals floor followed by conversion.
-__device__ __forceinline__ uint32_t quant(float v, float lo, float hi) {
-  v = fminf(fmaxf(v, lo), hi);
-  return __float2uint_rd(fadd(v, 0.5f));
+// Integers below 2^23 as the low bits of the binary32 number 2^23 + i: an
+// addition of 2^23, rounded down, is the floor of the other operand, and a
+// subtraction gives the integer as a number, both exact.  A conversion
+// instruction takes several times an addition's latency, and the conversions
+// of the prediction and the measurement lie one after the other in the model
+// chain (decode kernel 41.3 -> 39.9 us for 2000 tracks; no change where all
+// warps are resident).
+constexpr uint32_t kIntBits = 0x4B000000u;  // 2^23
+constexpr float kIntBase = 8388608.0f;
+
+// Quantiser: clamp to [0, hi] (NaN to 0), then floor(v + 0.5), as kIntBits + q.
+// fmaxf returns its non-NaN operand, so NaN clamps to 0; v + 0.5 then lies in
+// [0.5, hi + 0.5], below 2^23.
+__device__ __forceinline__ uint32_t quant(float v, float hi) {
+  v = fminf(fmaxf(v, 0.0f), hi);
+  return __float_as_uint(__fadd_rd(fadd(v, 0.5f), kIntBase));
 }
 
 struct Track {
@@ -124,10 +133,14 @@ struct Track {
 // y of a pad code on a row with geometry G = {x, w, 1/w, nPads/2}:
 // (pad / 64 - nPads/2) * w.
 __device__ __forceinline__ float pad_to_y(const float4& G, uint32_t padq) {
-  return fmul(ffma((float)padq, 0.015625f, -G.w), G.y);
+  const float p = fsub(__uint_as_float(kIntBits | padq), kIntBase);  // padq < 2^16
+  return fmul(ffma(p, 0.015625f, -G.w), G.y);
 }
+// Any 32-bit time code: its halves as numbers and one rounding.
 __device__ __forceinline__ float time_to_t(uint32_t timeq) {
-  return fmul((float)timeq, 0.03125f);
+  const float lo = fsub(__uint_as_float(__byte_perm(timeq, kIntBits, 0x7610)), kIntBase);
+  const float hi = fsub(__uint_as_float(__byte_perm(timeq, kIntBits, 0x7632)), kIntBase);
+  return fmul(ffma(hi, 65536.0f, lo), 0.03125f);
 }
 
 __device__ __forceinline__ void reset_ycov(Track& s) {
@@ -238,8 +251,8 @@ __device__ __forceinline__ void propagate_predict(const float4& G, Track& s, uin
   s.d01 = e1;
   s.d11 = ffma(kQTT, adx, s.d11);
   const float pp = ffma(s.y, G.z, G.w);
-  ppad = quant(fmul(pp, 64.0f), 0.0f, kPadHi);
-  ptime = quant(fmul(s.t, 32.0f), 0.0f, kTimeHi);
+  ppad = quant(fmul(pp, 64.0f), kPadHi) - kIntBits;
+  ptime = quant(fmul(s.t, 32.0f), kTimeHi) - kIntBits;
 }
 
 // Kalman update with the measured cluster (G: geometry of the current row).
