@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(256, 4) k_unatt_decode(const FrameDev* frames,
   __shared__ __align__(16) uint32_t s_stage[kStageWords];
   // the frame's unattached bin starts: every chunk searches them for the bins
   // of its clusters (loaded when a block's chunk comes from another frame)
-  __shared__ uint32_t s_ustart[kNBin + 1];
+  __shared__ __align__(16) uint32_t s_ustart[kNBin + 1];
   uint32_t* const s_rec = s_stage;                                  // variant 0
   uint32_t* const s_pos = s_stage + kRecWords + kRecWords / 32;     // variant 0
   uint4* const s_rec4 = reinterpret_cast<uint4*>(s_stage);          // variant 1
@@ -111,7 +111,18 @@ __global__ void __launch_bounds__(256, 4) k_unatt_decode(const FrameDev* frames,
       continue;
     }
     if (f != cached_f) {  // the same for every thread of the block
-      for (uint32_t i = tid; i <= (uint32_t)kNBin; i += blockDim.x) s_ustart[i] = F.unatt_start[i];
+      // 16-byte loads, all in flight (one by one they were half of the time of
+      // a block that decodes a single chunk)
+      constexpr int Q = (kNBin / 4 + 255) / 256;
+      const uint4* src = reinterpret_cast<const uint4*>(F.unatt_start);
+      uint4 v[Q];
+#pragma unroll
+      for (int q = 0; q < Q; q++)
+        if (tid + 256 * q < kNBin / 4) v[q] = src[tid + 256 * q];
+#pragma unroll
+      for (int q = 0; q < Q; q++)
+        if (tid + 256 * q < kNBin / 4) reinterpret_cast<uint4*>(s_ustart)[tid + 256 * q] = v[q];
+      if (tid == 0) s_ustart[kNBin] = F.unatt_start[kNBin];
       cached_f = f;
       __syncthreads();
     }
