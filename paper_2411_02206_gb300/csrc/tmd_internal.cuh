@@ -205,6 +205,5 @@ __global__ void k_track_trace(const FrameDev* frames, const uint32_t* ids, uint3
                               float* state);
 
 constexpr int kRankTags = 2048;  // per-warp duplicate-test slots of the ranking (bytes)
-constexpr int kRankGroup = 2;    // ranking steps tested for distinct keys at once
 
 }  // namespace tmd

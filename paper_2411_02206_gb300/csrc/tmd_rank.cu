@@ -36,15 +36,16 @@ namespace tmd {
 template <int W>
 constexpr int kRankSmem = W * (kNBin * 2 + kRankTags);
 
-// W warps per tile: 8 with two blocks per SM, or 16 when the call has no more
-// tiles than SMs (a warp's clusters are one serial chain: 20 us with 8 warps
-// for a frame of 190 k clusters, 18 us with 16).
-template <int W>
+// W warps per tile and G steps of 32 clusters tested for distinct keys at once:
+// 8 and 2 with two blocks per SM, or 16 and 4 when the call has no more tiles
+// than SMs (a warp's clusters are one serial chain: 20 us with 8 warps for a
+// frame of 190 k clusters, 17 us with 16).
+template <int W, int G>
 __global__ void __launch_bounds__(32 * W, 16 / W) k_count_rank(const FrameDev* frames, PlanDev plan,
                                                             bool sum) {
   // [W][kNBin/2] packed u16 counts, then [W][kRankTags] byte slots
-  constexpr int kTileWarps = W, kTileSub = kTile / W;
-  extern __shared__ uint32_t s_mem[];
+  constexpr int kTileWarps = W, kTileSub = kTile / W, kRankGroup = G;
+  extern __shared__ __align__(16) uint32_t s_mem[];
   const uint32_t f = find_frame(plan.pre_tile, plan.n_frames, blockIdx.x);
   const FrameDev& F = frames[f];
   if (*F.status & kStCount) return;
@@ -57,7 +58,9 @@ __global__ void __launch_bounds__(32 * W, 16 / W) k_count_rank(const FrameDev* f
   uint32_t* hist32 = s_mem + wid * (kNBin / 2);
   uint16_t* hist = reinterpret_cast<uint16_t*>(hist32);
   uint8_t* tag = reinterpret_cast<uint8_t*>(s_mem + kTileWarps * (kNBin / 2)) + wid * kRankTags;
-  for (int i = lane; i < kNBin / 2; i += 32) hist32[i] = 0u;
+  static_assert(kNBin % 8 == 0, "counters of a warp in 16-byte units");
+  for (int i = lane; i < kNBin / 8; i += 32)
+    reinterpret_cast<uint4*>(hist32)[i] = make_uint4(0u, 0u, 0u, 0u);
   __syncwarp();
   const uint32_t j_begin = tile * (uint32_t)kTile + wid * (uint32_t)kTileSub;
   const uint32_t j_end = min(j_begin + (uint32_t)kTileSub, n_att);
@@ -89,18 +92,22 @@ __global__ void __launch_bounds__(32 * W, 16 / W) k_count_rank(const FrameDev* f
     }
   }
   __syncthreads();
-  // per-warp exclusive offsets within the tile; tile histogram
-  uint16_t* hall = reinterpret_cast<uint16_t*>(s_mem);
-  for (int b = threadIdx.x; b < kNBin; b += blockDim.x) {
-    uint32_t run = 0;
+  // per-warp exclusive offsets within the tile, two bins per word (a tile's
+  // counts stay below 2^16); tile histogram
+  uint32_t* hist_o = reinterpret_cast<uint32_t*>(tile_hist + (size_t)tile * kNBin);
+#pragma unroll 2
+  for (int b = threadIdx.x; b < kNBin / 2; b += 32 * W) {
+    uint32_t c[W], run = 0;
 #pragma unroll
-    for (int ww = 0; ww < kTileWarps; ww++) {
-      const uint32_t c = hall[ww * kNBin + b];
-      hall[ww * kNBin + b] = (uint16_t)run;
-      run += c;
+    for (int ww = 0; ww < W; ww++) c[ww] = s_mem[ww * (kNBin / 2) + b];
+#pragma unroll
+    for (int ww = 0; ww < W; ww++) {
+      s_mem[ww * (kNBin / 2) + b] = run;
+      run += c[ww];
     }
-    tile_hist[(size_t)tile * kNBin + b] = (uint16_t)run;
-    if (sum && run) atomicAdd(&F.att_count[b], run);
+    hist_o[b] = run;
+    if (sum && (run & 0xFFFFu)) atomicAdd(&F.att_count[2 * b], run & 0xFFFFu);
+    if (sum && (run >> 16)) atomicAdd(&F.att_count[2 * b + 1], run >> 16);
   }
   __syncthreads();
   // pass 2: stable ranks in stream order; the keys of the next 8 steps are
@@ -194,16 +201,16 @@ __global__ void __launch_bounds__(32 * W, 16 / W) k_count_rank(const FrameDev* f
 void launch_count_rank(uint32_t n_tiles, bool sum, uint32_t sms, cudaStream_t st,
                        const FrameDev* frames, PlanDev plan) {
   if (n_tiles <= sms)
-    k_count_rank<16><<<n_tiles, 512, kRankSmem<16>, st>>>(frames, plan, sum);
+    k_count_rank<16, 4><<<n_tiles, 512, kRankSmem<16>, st>>>(frames, plan, sum);
   else
-    k_count_rank<8><<<n_tiles, 256, kRankSmem<8>, st>>>(frames, plan, sum);
+    k_count_rank<8, 2><<<n_tiles, 256, kRankSmem<8>, st>>>(frames, plan, sum);
 }
 
 cudaError_t prepare_count_rank() {
-  cudaError_t e = cudaFuncSetAttribute(k_count_rank<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(k_count_rank<8, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kRankSmem<8>);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_count_rank<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(k_count_rank<16, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kRankSmem<16>);
   return e;
 }
