@@ -204,13 +204,16 @@ __device__ __forceinline__ void sector_change(const RowGeo* g, Track& s, int sd)
   reset_ycov(s);
 }
 
-// Key step of one cluster: row and sector/leg differences.  A row outside the
-// detector shows in s.max_row.
-__device__ __forceinline__ void key_step(const RowGeo* g, Track& s, uint32_t row_diff,
-                                         uint32_t sld) {
-  s.raw_row = (s.raw_row + (int)row_diff) & 255;
-  s.max_row = max(s.max_row, s.raw_row);
-  s.row = min(s.raw_row, kNRow - 1);
+// Key step of one cluster in its two parts: the row, which no decoded
+// coordinate enters (raw: the row walk's new value, mod 256; a row outside the
+// detector shows in s.max_row), and the sector/leg difference.
+__device__ __forceinline__ int clamp_row(int raw) { return min(raw, kNRow - 1); }
+__device__ __forceinline__ void row_step(Track& s, int raw) {
+  s.raw_row = raw;
+  s.max_row = max(s.max_row, raw);
+  s.row = clamp_row(raw);
+}
+__device__ __forceinline__ void turn_step(const RowGeo* g, Track& s, uint32_t sld) {
   if (sld != 0) {  // few clusters
     uint32_t sd = sld;
     if (sld >= (uint32_t)kNSec) {
