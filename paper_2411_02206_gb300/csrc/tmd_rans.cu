@@ -309,28 +309,49 @@ __device__ uint64_t check_entry(const Job& J, const JobField& F, uint32_t w) {
 // steps earlier at the latest.
 struct Words {
   uint32_t ring;         // shared-memory address of the lane's first pair
-  const uint32_t* next;  // pair number `queued`
+  uint64_t next;         // address of pair number `queued`
   uint32_t queued, have; // pairs queued, pairs there are
   uint32_t used;         // words used
   uint32_t w0, w1;       // the next four words, the first one lowest
 
-  // past the chunk's last pair nothing is copied: a stream that reads on is
-  // found by its count of words
-  __device__ __forceinline__ void queue() {
-    if (queued < have) {
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(ring + (queued % kRing) * 128),
-                   "l"(next) : "memory");
-      next += 32;
-    }
-    queued++;
+  // Queues the next pair if fewer than `upto` are.  Past the chunk's last pair
+  // nothing is copied: a stream that reads on is found by its count of words.
+  // Predicated by hand, like refill: as branches the two cost a warp, most of
+  // whose lanes take them at most symbols, half of its instructions.
+  __device__ __forceinline__ void queue(uint32_t upto) {
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p, q;\n\t"
+        "setp.lt.u32 p, %1, %2;\n\t"
+        "setp.lt.and.u32 q, %1, %3, p;\n\t"
+        "@q cp.async.ca.shared.global [%4], [%0], 4;\n\t"
+        "@q add.u64 %0, %0, 128;\n\t"
+        "@p add.u32 %1, %1, 1;\n\t"
+        "}"
+        : "+l"(next), "+r"(queued)
+        : "r"(upto), "r"(have), "r"(ring + (queued % kRing) * 128)
+        : "memory");
+  }
+  // The state's refill with the next word, if it fell below the interval.
+  __device__ __forceinline__ void refill(uint32_t& x) {
+    static_assert(kLower == 65536, "");
+    asm("{\n\t"
+        ".reg .pred p;\n\t"
+        "setp.lt.u32 p, %0, 65536;\n\t"
+        "@p prmt.b32 %0, %1, %0, 0x5410;\n\t"
+        "@p prmt.b32 %1, %1, %2, 0x5432;\n\t"
+        "@p shr.u32 %2, %2, 16;\n\t"
+        "@p add.u32 %3, %3, 1;\n\t"
+        "}"
+        : "+r"(x), "+r"(w0), "+r"(w1), "+r"(used));
   }
   __device__ __forceinline__ void start(uint32_t ring_, const uint32_t* first, uint32_t n) {
     ring = ring_;
-    next = first;
+    next = reinterpret_cast<uint64_t>(first);
     have = n;
     queued = used = 0;
 #pragma unroll
-    for (uint32_t i = 0; i < kRing; i++) queue();
+    for (uint32_t i = 0; i < kRing; i++) queue(kRing);
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
   }
   __device__ __forceinline__ uint32_t pair(uint32_t row) const {
@@ -342,7 +363,7 @@ struct Words {
     static_assert(kRing == 8, "see above");
 #pragma unroll
     for (int i = 0; i < 2; i++)
-      if (queued < used / 2 + kRing) queue();
+      queue(used / 2 + kRing);
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 2;" ::: "memory");
     const uint32_t row = used * 64, sh = used % 2 * 16;
     const uint32_t a = pair(row), b = pair(row + 128), c = pair(row + 256);
@@ -450,12 +471,7 @@ __device__ __forceinline__ void decode_block(const Job& J, const JobField& F, ui
           const uint32_t xs = x >> 12;
           x = ((e >> 8) & (kM - 1)) * xs + xs + (e >> 20);
           v = __byte_perm(v, e, p == 0 ? 0x3214 : p == 1 ? 0x3240 : p == 2 ? 0x3410 : 0x4210);
-          if (x < kLower) {
-            x = __byte_perm(words.w0, x, 0x5410);
-            words.w0 = __byte_perm(words.w0, words.w1, 0x5432);
-            words.w1 >>= 16;
-            words.used++;
-          }
+          words.refill(x);
           low = min(low, x);
         }
         return (T)v;
