@@ -548,11 +548,13 @@ int tmd_enqueue(tmd_handle* h, uint32_t nf, const tmd_frame_in* in, const tmd_fr
     most_tiles = std::max(most_tiles, fd[f].n_tiles);
   }
   if (most_tracks <= (uint32_t)kPrepTracks) {
-    timed(kKTrackPrep, [&] { k_track_prep<<<dim3(nf, 2), 1024, 0, st>>>(dframes); });
+    timed(kKTrackPrep, [&] { launch_chained(k_track_prep, dim3(nf, 2), 1024, 0, st, dframes); });
   } else {
-    if (n_tblk) timed(kKTrackScan1, [&] { k_track_scan1<<<n_tblk, 256, 0, st>>>(dframes, P); });
-    timed(kKFrameScan, [&] { k_frame_scan<<<nf, 1024, 0, st>>>(dframes, P); });
-    if (n_tblk) timed(kKTrackScan2, [&] { k_track_scan2<<<n_tblk, 256, 0, st>>>(dframes, P); });
+    if (n_tblk)
+      timed(kKTrackScan1, [&] { launch_chained(k_track_scan1, n_tblk, 256, 0, st, dframes, P); });
+    timed(kKFrameScan, [&] { launch_chained(k_frame_scan, nf, 1024, 0, st, dframes, P); });
+    if (n_tblk)
+      timed(kKTrackScan2, [&] { launch_chained(k_track_scan2, n_tblk, 256, 0, st, dframes, P); });
   }
   if (trace) {
     if (trace->n)
@@ -600,8 +602,8 @@ int tmd_enqueue(tmd_handle* h, uint32_t nf, const tmd_frame_in* in, const tmd_fr
     if (n_tile)
       timed(kKCountRank, [&] { launch_count_rank(n_tile, !groups, (uint32_t)h->sms, st, dframes, P); });
     if (groups)
-      timed(kKGroupSum, [&] { k_group_sum<<<n_grp, kBinBlk, 0, st>>>(dframes, P); });
-    timed(kKRowOffsets, [&] { k_row_offsets<<<nf, 1024, 0, st>>>(dframes, P); });
+      timed(kKGroupSum, [&] { launch_chained(k_group_sum, n_grp, kBinBlk, 0, st, dframes, P); });
+    timed(kKRowOffsets, [&] { launch_chained(k_row_offsets, nf, 1024, 0, st, dframes, P); });
     auto unatt = [&](cudaStream_t s_) {
       if (!n_chunk) return;
       // beside the scatter the tuned number of blocks per SM; alone, every
@@ -611,7 +613,7 @@ int tmd_enqueue(tmd_handle* h, uint32_t nf, const tmd_frame_in* in, const tmd_fr
       if (s_ != st && h->tune_unatt_bps > 0 && h->tune_unatt_bps < bps) bps = h->tune_unatt_bps;
       const uint32_t grid = std::min<uint32_t>(n_chunk, (uint32_t)(h->sms * bps));
       timed_on(s_, kKUnattDecode, [&] {
-        launch_unatt_decode(h->tune_unatt_variant, grid, s_, dframes, P, n_chunk);
+        launch_unatt_decode(h->tune_unatt_variant, grid, s_, dframes, P, n_chunk, s_ == st && n_tile);
       });
     };
     if (cs && cs->late) CK(cudaStreamWaitEvent(st, cs->late, 0));
@@ -620,7 +622,12 @@ int tmd_enqueue(tmd_handle* h, uint32_t nf, const tmd_frame_in* in, const tmd_fr
       CK(cudaStreamWaitEvent(cs->aux, cs->fork, 0));
       unatt(cs->aux);
     }
-    if (n_grp) timed(kKTileBase, [&] { k_tile_base<<<n_grp, kBinBlk, 0, st>>>(dframes, P); });
+    // after an event the tile bases are launched plainly
+    if (n_grp)
+      timed(kKTileBase, [&] {
+        if (two || (cs && cs->late)) k_tile_base<<<n_grp, kBinBlk, 0, st>>>(dframes, P);
+        else launch_chained(k_tile_base, n_grp, kBinBlk, 0, st, dframes, P);
+      });
     if (n_tile)
       timed(kKAttScatter, [&] { launch_att_scatter(h->tune_scatter_variant, n_tile, st, dframes, P); });
     if (two) {

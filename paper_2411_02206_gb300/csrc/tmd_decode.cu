@@ -152,6 +152,7 @@ __global__ void __launch_bounds__(kDecodeThreads, MINB)
   __shared__ RowGeo geo_s;
   extern __shared__ __align__(16) uint32_t s_stage[];
   fill_row_geo(&geo_s);
+  chain_wait();
   __syncthreads();
   const RowGeo* geo = &geo_s;
   const uint32_t lane = threadIdx.x & 31, lanes = plan.lanes;
@@ -309,9 +310,11 @@ constexpr int kDecodeSmem = (kDecodeThreads / 32) * (int)sizeof(AsyncStage<R>);
 void launch_track_decode(int variant, uint32_t grid, cudaStream_t st, const FrameDev* frames,
                          PlanDev plan, uint32_t n_tasks) {
   if (variant == 1)
-    k_track_decode<8, 5><<<grid, kDecodeThreads, kDecodeSmem<8>, st>>>(frames, plan, n_tasks);
+    launch_chained(k_track_decode<8, 5>, grid, kDecodeThreads, kDecodeSmem<8>, st, frames,
+                   plan, n_tasks);
   else
-    k_track_decode<16, 3><<<grid, kDecodeThreads, kDecodeSmem<16>, st>>>(frames, plan, n_tasks);
+    launch_chained(k_track_decode<16, 3>, grid, kDecodeThreads, kDecodeSmem<16>, st, frames,
+                   plan, n_tasks);
 }
 
 cudaError_t prepare_track_decode(int variant, int* blocks_per_sm) {
@@ -435,6 +438,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 3)
   __shared__ RowGeo geo;
   extern __shared__ __align__(16) uint32_t s_stage[];
   fill_row_geo(&geo);
+  chain_wait();
   __syncthreads();
   EncStage& S = reinterpret_cast<EncStage*>(s_stage)[threadIdx.x >> 5];
   const uint32_t lane = threadIdx.x & 31, lanes = plan.lanes;
@@ -585,7 +589,8 @@ constexpr int kEncodeSmem = (kDecodeThreads / 32) * (int)sizeof(EncStage);
 
 void launch_track_encode(uint32_t grid, cudaStream_t st, const EncDev* enc, const FrameDev* frames,
                          PlanDev plan, uint32_t n_tasks) {
-  k_track_encode<<<grid, kDecodeThreads, kEncodeSmem, st>>>(enc, frames, plan, n_tasks);
+  launch_chained(k_track_encode, grid, kDecodeThreads, kEncodeSmem, st, enc, frames, plan,
+                 n_tasks);
 }
 
 cudaError_t prepare_track_encode(int* blocks_per_sm) {

@@ -46,6 +46,7 @@ __global__ void __launch_bounds__(32 * W, 16 / W) k_count_rank(const FrameDev* f
   // [W][kNBin/2] packed u16 counts, then [W][kRankTags] byte slots
   constexpr int kTileWarps = W, kTileSub = kTile / W, kRankGroup = G;
   extern __shared__ __align__(16) uint32_t s_mem[];
+  chain_wait();
   const uint32_t f = find_frame(plan.pre_tile, plan.n_frames, blockIdx.x);
   const FrameDev& F = frames[f];
   if (*F.status & kStCount) return;
@@ -201,9 +202,9 @@ __global__ void __launch_bounds__(32 * W, 16 / W) k_count_rank(const FrameDev* f
 void launch_count_rank(uint32_t n_tiles, bool sum, uint32_t sms, cudaStream_t st,
                        const FrameDev* frames, PlanDev plan) {
   if (n_tiles <= sms)
-    k_count_rank<16, 4><<<n_tiles, 512, kRankSmem<16>, st>>>(frames, plan, sum);
+    launch_chained(k_count_rank<16, 4>, n_tiles, 512, kRankSmem<16>, st, frames, plan, sum);
   else
-    k_count_rank<8, 2><<<n_tiles, 256, kRankSmem<8>, st>>>(frames, plan, sum);
+    launch_chained(k_count_rank<8, 2>, n_tiles, 256, kRankSmem<8>, st, frames, plan, sum);
 }
 
 cudaError_t prepare_count_rank() {

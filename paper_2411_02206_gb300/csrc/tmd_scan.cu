@@ -124,6 +124,7 @@ __global__ void k_zero_status(const FrameDev* frames, uint32_t n_frames) {
 
 // Block totals of the track lengths, zero-length check, length histogram.
 __global__ void __launch_bounds__(256) k_track_scan1(const FrameDev* frames, PlanDev plan) {
+  chain_wait();
   __shared__ uint32_t hist[kLenBuckets];
   uint32_t tot;
   const uint32_t f = find_frame(plan.pre_tblk, plan.n_frames, blockIdx.x);
@@ -182,6 +183,7 @@ __device__ __forceinline__ void unatt_bins(const FrameDev& F) {
 // Per frame: offsets of the track blocks, decode-order bucket offsets (longest
 // first), unattached bin starts, count checks.
 __global__ void __launch_bounds__(1024) k_frame_scan(const FrameDev* frames, PlanDev plan) {
+  chain_wait();
   uint32_t tot;
   const FrameDev& F = frames[blockIdx.x];
   const uint32_t tid = threadIdx.x;
@@ -208,6 +210,7 @@ __global__ void __launch_bounds__(1024) k_frame_scan(const FrameDev* frames, Pla
 // one global atomic per bucket; the order of tracks of equal length is
 // arbitrary (it only changes which warp decodes a track, not a result).
 __global__ void __launch_bounds__(256) k_track_scan2(const FrameDev* frames, PlanDev plan) {
+  chain_wait();
   __shared__ uint32_t s_cnt[kLenBuckets];
   uint32_t tot;
   const uint32_t f = find_frame(plan.pre_tblk, plan.n_frames, blockIdx.x);
@@ -255,6 +258,7 @@ __global__ void __launch_bounds__(256) k_track_scan2(const FrameDev* frames, Pla
 // for 2000 tracks where this one takes 8 us.
 __global__ void __launch_bounds__(1024) k_track_prep(const FrameDev* frames) {
   __shared__ uint32_t s_cur[kLenBuckets];
+  chain_wait();
   const FrameDev& F = frames[blockIdx.x];
   if (blockIdx.y == 1) {
     unatt_bins(F);
@@ -306,6 +310,7 @@ __global__ void __launch_bounds__(1024) k_track_prep(const FrameDev* frames) {
 // sums are also added into the bin's attached count (cleared by k_frame_scan).
 // Calls with a frame of several groups; see launch_count_rank.
 __global__ void __launch_bounds__(kBinBlk) k_group_sum(const FrameDev* frames, PlanDev plan) {
+  chain_wait();
   const uint32_t f = find_frame(plan.pre_grp, plan.n_frames, blockIdx.x);
   const FrameDev& F = frames[f];
   if (*F.status & kStCount) return;
@@ -347,6 +352,7 @@ __device__ __forceinline__ void row_start_scan(const FrameDev& F) {
 
 // Per frame: rowStart (the attached counts are there).
 __global__ void __launch_bounds__(1024) k_row_offsets(const FrameDev* frames, PlanDev plan) {
+  chain_wait();
   const FrameDev& F = frames[blockIdx.x];
   if (*F.status & kStCount) return;
   row_start_scan(F);
@@ -355,6 +361,7 @@ __global__ void __launch_bounds__(1024) k_row_offsets(const FrameDev* frames, Pl
 // First native index of every (tile, bin): rowStart plus the counts of the
 // bin in the groups and tiles before.
 __global__ void __launch_bounds__(kBinBlk) k_tile_base(const FrameDev* frames, PlanDev plan) {
+  chain_wait();
   const uint32_t f = find_frame(plan.pre_grp, plan.n_frames, blockIdx.x);
   const FrameDev& F = frames[f];
   if (*F.status & kStCount) return;

@@ -26,6 +26,7 @@ namespace tmd {
 template <int V, int U>
 __global__ void __launch_bounds__(kScatThreads, 4) k_att_scatter(const FrameDev* frames,
                                                                  PlanDev plan) {
+  chain_wait();
   constexpr uint32_t kPerBlock = kScatThreads * U;
   constexpr uint32_t kBlocksPerTile = kTile / kPerBlock;
   const uint32_t gtile = blockIdx.x / kBlocksPerTile;
@@ -111,9 +112,9 @@ void launch_att_scatter(int variant, uint32_t n_tiles, cudaStream_t st, const Fr
                         PlanDev plan) {
   const uint32_t grid = n_tiles * (kTile / (kScatThreads * 4));
   if (variant == 0)
-    k_att_scatter<0, 4><<<grid, kScatThreads, 0, st>>>(frames, plan);
+    launch_chained(k_att_scatter<0, 4>, grid, kScatThreads, 0, st, frames, plan);
   else
-    k_att_scatter<1, 4><<<grid, kScatThreads, 0, st>>>(frames, plan);
+    launch_chained(k_att_scatter<1, 4>, grid, kScatThreads, 0, st, frames, plan);
 }
 
 }  // namespace tmd

@@ -84,6 +84,7 @@ __device__ __forceinline__ uint32_t rec4_slot(uint32_t l) { return l ^ ((l >> 3)
 template <int V>
 __global__ void __launch_bounds__(256, 4) k_unatt_decode(const FrameDev* frames, PlanDev plan,
                                                       uint32_t n_tickets) {
+  chain_wait();
   constexpr uint32_t kRecWords = 3 * kChunk;
   constexpr uint32_t kStageWords = V == 0 ? kRecWords + kRecWords / 32 + kChunk : 4 * kChunk;
   __shared__ uint32_t s_ticket;
@@ -340,11 +341,12 @@ __global__ void __launch_bounds__(256, 4) k_unatt_decode(const FrameDev* frames,
 }
 
 void launch_unatt_decode(int variant, uint32_t grid, cudaStream_t st, const FrameDev* frames,
-                         PlanDev plan, uint32_t n_tickets) {
-  if (variant == 1)
-    k_unatt_decode<1><<<grid, 256, 0, st>>>(frames, plan, n_tickets);
+                         PlanDev plan, uint32_t n_tickets, bool chained) {
+  const auto kern = variant == 1 ? k_unatt_decode<1> : k_unatt_decode<0>;
+  if (chained)
+    launch_chained(kern, grid, 256, 0, st, frames, plan, n_tickets);
   else
-    k_unatt_decode<0><<<grid, 256, 0, st>>>(frames, plan, n_tickets);
+    kern<<<grid, 256, 0, st>>>(frames, plan, n_tickets);
 }
 
 cudaError_t occupancy_unatt_decode(int* blocks_per_sm) {

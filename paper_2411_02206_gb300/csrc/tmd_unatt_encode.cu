@@ -115,6 +115,7 @@ __global__ void __launch_bounds__(256) k_ue_init(UeArgs a, UeCtl* ctl) {
 // Clusters per bin: counters in shared memory, added to the output once per
 // block (so a block takes at least a few thousand clusters).
 __global__ void __launch_bounds__(1024) k_ue_count(UeArgs a) {
+  chain_wait();
   __shared__ uint32_t s_cnt[kNBin];
   for (int i = threadIdx.x; i < kNBin; i += 1024) s_cnt[i] = 0u;
   __syncthreads();
@@ -167,6 +168,7 @@ __device__ __forceinline__ uint32_t ue_scan(uint32_t v, uint32_t& tot) {
 
 // One block: output positions of the bins, and which kernel sorts each.
 __global__ void __launch_bounds__(1024) k_ue_plan(UeArgs a, UePlan* plan, UeCtl* ctl) {
+  chain_wait();
   constexpr int Q = (kNBin + 1023) / 1024;
   const uint32_t b0 = threadIdx.x * Q;
   uint32_t v[Q], sum = 0, tot;
@@ -207,6 +209,7 @@ __global__ void __launch_bounds__(1024) k_ue_plan(UeArgs a, UePlan* plan, UeCtl*
 // counters, makes every reservation a request of its own: 442 us.
 __global__ void __launch_bounds__(kUeScatThreads, 3) k_ue_scatter(UeArgs a, uint4* __restrict__ rec,
                                                                  UePlan* plan, UeCtl* ctl) {
+  chain_wait();
   constexpr int T = kUeScatThreads;
   __shared__ __align__(16) uint32_t s_cnt[kNBin];
   const uint32_t tid = threadIdx.x;
@@ -301,6 +304,7 @@ __device__ __forceinline__ uint64_t ue_key(uint32_t x, uint32_t y) {
 // of its records, the records that come before it.
 __global__ void __launch_bounds__(256) k_ue_sort_warp(UeArgs a, const uint4* __restrict__ rec,
                                                      const UePlan* plan, const UeCtl* ctl) {
+  chain_wait();
   constexpr int E = kUeWarpMax / 32;
   __shared__ uint4 s_rec[8][kUeWarpMax];
   __shared__ uint8_t s_ord[8][kUeWarpMax];
@@ -413,6 +417,7 @@ __device__ __forceinline__ void ue_minmax(uint32_t& lo, uint32_t& hi, uint32_t* 
 __global__ void __launch_bounds__(kUeBlockThreads, 3) k_ue_sort_block(UeArgs a, const uint4* rec,
                                                                      const UePlan* plan,
                                                                      UeCtl* ctl) {
+  chain_wait();
   constexpr int T = kUeBlockThreads, E = kUeBlockMax / T;
   extern __shared__ uint64_t s_dyn[];
   uint64_t* s_key = s_dyn;                                            // kUeBlockMax
@@ -493,6 +498,7 @@ __global__ void __launch_bounds__(kUeBlockThreads, 3) k_ue_sort_block(UeArgs a, 
 // of about kUeSliceMean clusters, sorted and written one after the other.
 __global__ void __launch_bounds__(kUeBigThreads, 1) k_ue_sort_big(UeArgs a, const uint4* rec,
                                                                  const UePlan* plan, UeCtl* ctl) {
+  chain_wait();
   constexpr int T = kUeBigThreads, E = kUeSliceCap / T;
   extern __shared__ uint64_t s_dyn[];
   uint64_t* s_key = s_dyn;                                            // kUeSliceCap
@@ -844,17 +850,17 @@ extern "C" int tmd_encode_unattached(tmd_handle* h, const tmd_unatt_truth_in* in
   const uint32_t sms = (uint32_t)h->sms;
   k_ue_init<<<(kNBin + 9 + 255) / 256, 256, 0, st>>>(a, ctl);
   if (n) {
-    k_ue_count<<<std::min(2 * sms, n / 8192 + 1), 1024, 0, st>>>(a);
-    k_ue_plan<<<1, 1024, 0, st>>>(a, plan, ctl);
-    k_ue_scatter<<<n / (kUeScatThreads * 4) + (n % (kUeScatThreads * 4) != 0), kUeScatThreads, 0,
-                   st>>>(a, r0, plan, ctl);
-    k_ue_sort_warp<<<(kNBin + 7) / 8, 256, 0, st>>>(a, r0, plan, ctl);
+    launch_chained(k_ue_count, std::min(2 * sms, n / 8192 + 1), 1024, 0, st, a);
+    launch_chained(k_ue_plan, 1, 1024, 0, st, a, plan, ctl);
+    launch_chained(k_ue_scatter, n / (kUeScatThreads * 4) + (n % (kUeScatThreads * 4) != 0),
+                   kUeScatThreads, 0, st, a, r0, plan, ctl);
+    launch_chained(k_ue_sort_warp, (kNBin + 7) / 8, 256, 0, st, a, r0, plan, ctl);
     if (n > kUeWarpMax)
-      k_ue_sort_block<<<std::min(3 * sms, n / kUeWarpMax), kUeBlockThreads, kUeBlockSmem, st>>>(
-          a, r0, plan, ctl);
+      launch_chained(k_ue_sort_block, std::min(3 * sms, n / kUeWarpMax), kUeBlockThreads,
+                     kUeBlockSmem, st, a, r0, plan, ctl);
     if (n > kUeBlockMax)
-      k_ue_sort_big<<<std::min(sms, n / kUeBlockMax), kUeBigThreads, kUeBigSmem, st>>>(a, r0, plan,
-                                                                                    ctl);
+      launch_chained(k_ue_sort_big, std::min(sms, n / kUeBlockMax), kUeBigThreads, kUeBigSmem, st,
+                     a, r0, plan, ctl);
     void* args[] = {&a, &r0, &r1, &plan, &ctl, &cnt, &dig};
     const uint32_t grid = std::min(n_tiles, sms * (uint32_t)h->occ_ue);
     rc = tmd_cuda_check(h, cudaLaunchCooperativeKernel((const void*)k_ue_general, dim3(grid),
