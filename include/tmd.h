@@ -300,11 +300,12 @@ typedef struct tmd_unatt_out {
  * sorted by (time, pad) ascending with ties in input order; pad_diff_u /
  * time_diff_u = the cluster's pad / time minus those of the preceding
  * cluster of its bin (the first of a bin minus 0), mod 2^16 / 2^32; charges,
- * flags and sigmas in the same order; n_unatt = clusters per bin.  Stable
- * LSD radix sort on the GPU, asynchronous on `stream`, handle scratch of
- * about 24 bytes per cluster.  *status receives TMD_STATUS_ROW if a row >=
- * 152 or a sector >= 36 (outputs then unspecified).  Errors: TMD_ERR_ARG
- * (null or misaligned pointer), TMD_ERR_NOMEM, TMD_ERR_CUDA. */
+ * flags and sigmas in the same order; n_unatt = clusters per bin.
+ * Asynchronous on `stream`; handle scratch of about 33 bytes per cluster.
+ * *status receives TMD_STATUS_ROW if a row >= 152 or a sector >= 36 and
+ * TMD_STATUS_TIMEOUT if a bounded wait inside the sort expired (outputs then
+ * unspecified).  Errors: TMD_ERR_ARG (null or misaligned pointer),
+ * TMD_ERR_NOMEM, TMD_ERR_CUDA. */
 int tmd_encode_unattached(tmd_handle* h, const tmd_unatt_truth_in* in, const tmd_unatt_out* out,
                           void* stream);
 
@@ -523,9 +524,11 @@ typedef struct tmd_coded_frame {
 /* The host streaming pipeline of tmd_decode_host_stream for coded frames, the
  * form in which the paper's compressed time frames cross the host link
  * (Sec. 4, Fig. 2): frame i's coded bytes go up in one copy on a copy stream
- * while earlier frames are entropy-decoded and track-model decoded (as by
- * tmd_decode_coded_frame) on `stream` and their results come back to out[]
- * on a second copy stream, through three handle-owned device slots.
+ * while earlier frames are entropy-decoded on a stream of the handle, one frame
+ * ahead of the track-model decoding on `stream`, into two handle-owned sets of
+ * streams (tuning key coded_overlap 0, a single frame, or no memory for two
+ * sets: on `stream`, as by tmd_decode_coded_frame), and their results come back
+ * to out[] on a second copy stream, through three handle-owned device slots.
  * Synchronous on return; results equal those of tmd_decode_coded_frame.
  * Errors: TMD_ERR_ARG (null pointer, n_attached < n_tracks, bytes <
  * TMD_RANS_HEADER_BYTES), TMD_ERR_NOMEM, TMD_ERR_CUDA. */

@@ -209,6 +209,12 @@ tmd_handle::~tmd_handle() {
   if (join) cudaEventDestroy(join);
   if (h2d) cudaStreamSynchronize(h2d), cudaStreamDestroy(h2d);
   if (d2h) cudaStreamSynchronize(d2h), cudaStreamDestroy(d2h);
+  if (ent) cudaStreamSynchronize(ent), cudaStreamDestroy(ent);
+  for (int b = 0; b < 2; b++) {
+    if (ent_buf[b]) cudaFree(ent_buf[b]);
+    for (cudaEvent_t e : {ent_done[b], ent_free[b]})
+      if (e) cudaEventDestroy(e);
+  }
   for (int s = 0; s < kPipeSlots; s++) {
     if (pipe_buf[s]) cudaFree(pipe_buf[s]);
     for (cudaEvent_t e : {pipe_in[s], pipe_dec[s], pipe_out[s]})

@@ -93,6 +93,12 @@ struct tmd_handle {
   void* pipe_buf[kPipeSlots] = {};
   size_t pipe_bytes[kPipeSlots] = {};
   cudaEvent_t pipe_in[kPipeSlots] = {}, pipe_dec[kPipeSlots] = {}, pipe_out[kPipeSlots] = {};
+  // coded frames: entropy decoding one frame ahead of the decode chain, into
+  // two sets of streams in turn
+  cudaStream_t ent = nullptr;
+  void* ent_buf[2] = {};
+  size_t ent_bytes[2] = {};
+  cudaEvent_t ent_done[2] = {}, ent_free[2] = {};
 
   // Calls share the scratch (and the coded-frame streams): a call on any
   // stream first waits for the previous call's work on them, recorded in
@@ -147,6 +153,13 @@ int tmd_enqueue(tmd_handle* h, uint32_t nf, const tmd_frame_in* in, const tmd_fr
                 const tmd_truth_in* tin, const tmd_track_out* tout, void* scratch,
                 void* host_record, void* dev_record, cudaStream_t st, bool profile,
                 const ChainStreams* cs = nullptr, const TraceReq* trace = nullptr);
+// The two halves of tmd_decode_coded_frame on a caller's buffer of
+// tmd_coded_stream_bytes: entropy decoding into it, and the decode chain from it.
+size_t tmd_coded_stream_bytes(uint32_t n_tracks, uint32_t n_attached, uint32_t n_unattached);
+int tmd_coded_entropy(tmd_handle* h, const tmd_coded_frame* in, const void* coded, void* streams,
+                      cudaStream_t st);
+int tmd_coded_chain(tmd_handle* h, const tmd_coded_frame* in, void* streams,
+                    const tmd_frame_out* out, cudaStream_t st);
 // Shared-memory attribute of the entropy decoder.
 cudaError_t prepare_rans_decode();
 void tmd_serve_shutdown(tmd_handle* h);

@@ -663,6 +663,80 @@ extern "C" int tmd_rans_decode(tmd_handle* h, const void* coded, uint64_t coded_
   return tmd_cuda_check(h, launch_streams(h, c, coded_bytes, *dst, status, st), "k_rans_decode");
 }
 
+namespace {
+
+// The entropy-decoded streams of a frame in one buffer: each array 256-byte
+// aligned, then a status word.
+tmd_frame_arrays coded_arrays(void* buf, uint32_t n_tracks, uint32_t n_attached,
+                              uint32_t n_unattached, uint32_t** status) {
+  uint8_t* b = static_cast<uint8_t*>(buf);
+  tmd_frame_arrays a;
+  a.n_tracks = n_tracks;
+  a.n_attached = n_attached;
+  a.n_unattached = n_unattached;
+  void** slots[kFields] = {
+      (void**)&a.qpt,      (void**)&a.row,         (void**)&a.slice,        (void**)&a.pad,
+      (void**)&a.time,     (void**)&a.ncl,         (void**)&a.qtot_a,       (void**)&a.qmax_a,
+      (void**)&a.flags_a,  (void**)&a.sigma_pad_a, (void**)&a.sigma_time_a, (void**)&a.row_diff,
+      (void**)&a.slice_leg_diff, (void**)&a.pad_res, (void**)&a.time_res,   (void**)&a.n_unatt,
+      (void**)&a.pad_diff_u, (void**)&a.time_diff_u, (void**)&a.qtot_u,     (void**)&a.qmax_u,
+      (void**)&a.flags_u,  (void**)&a.sigma_pad_u, (void**)&a.sigma_time_u};
+  size_t off = 0;
+  for (int f = 0; f < kFields; f++) {
+    *slots[f] = b + off;
+    off += ((size_t)field_len(f, n_tracks, n_attached, n_unattached) * kWidth[f] + 255) & ~size_t(255);
+  }
+  *status = reinterpret_cast<uint32_t*>(b + off);
+  return a;
+}
+
+tmd_frame_in frame_of(const tmd_frame_arrays& a) {
+  tmd_frame_in in;
+  in.n_tracks = a.n_tracks;
+  in.n_attached = a.n_attached;
+  in.n_unattached = a.n_unattached;
+  in.qpt = a.qpt; in.row = a.row; in.slice = a.slice; in.pad = a.pad; in.time = a.time;
+  in.ncl = a.ncl; in.qtot_a = a.qtot_a; in.qmax_a = a.qmax_a; in.flags_a = a.flags_a;
+  in.sigma_pad_a = a.sigma_pad_a; in.sigma_time_a = a.sigma_time_a; in.row_diff = a.row_diff;
+  in.slice_leg_diff = a.slice_leg_diff; in.pad_res = a.pad_res; in.time_res = a.time_res;
+  in.n_unatt = a.n_unatt; in.pad_diff_u = a.pad_diff_u; in.time_diff_u = a.time_diff_u;
+  in.qtot_u = a.qtot_u; in.qmax_u = a.qmax_u; in.flags_u = a.flags_u;
+  in.sigma_pad_u = a.sigma_pad_u; in.sigma_time_u = a.sigma_time_u;
+  return in;
+}
+
+}  // namespace
+
+size_t tmd_coded_stream_bytes(uint32_t n_tracks, uint32_t n_attached, uint32_t n_unattached) {
+  size_t total = 256;
+  for (int f = 0; f < kFields; f++)
+    total += ((size_t)field_len(f, n_tracks, n_attached, n_unattached) * kWidth[f] + 255) & ~size_t(255);
+  return total;
+}
+
+int tmd_coded_entropy(tmd_handle* h, const tmd_coded_frame* in, const void* coded, void* streams,
+                      cudaStream_t st) {
+  uint32_t* status = nullptr;
+  const tmd_frame_arrays a =
+      coded_arrays(streams, in->n_tracks, in->n_attached, in->n_unattached, &status);
+  const int rc = tmd_cuda_check(h, cudaMemsetAsync(status, 0, 4, st), "cudaMemsetAsync");
+  if (rc != TMD_OK) return rc;
+  return tmd_cuda_check(h, launch_streams(h, static_cast<const uint8_t*>(coded), in->bytes, a, status,
+                                          st), "k_rans_decode");
+}
+
+int tmd_coded_chain(tmd_handle* h, const tmd_coded_frame* in, void* streams,
+                    const tmd_frame_out* out, cudaStream_t st) {
+  uint32_t* status = nullptr;
+  const tmd_frame_arrays a =
+      coded_arrays(streams, in->n_tracks, in->n_attached, in->n_unattached, &status);
+  const tmd_frame_in fin = frame_of(a);
+  const int rc = tmd_decode_frame(h, &fin, out, st);
+  if (rc != TMD_OK) return rc;
+  k_status_or<<<1, 1, 0, st>>>(out->status, status);
+  return tmd_cuda_check(h, cudaGetLastError(), "k_status_or launch");
+}
+
 extern "C" int tmd_decode_coded_frame(tmd_handle* h, const void* coded, uint64_t coded_bytes,
                                       uint32_t n_tracks, uint32_t n_attached,
                                       uint32_t n_unattached, const tmd_frame_out* out,
@@ -674,14 +748,7 @@ extern "C" int tmd_decode_coded_frame(tmd_handle* h, const void* coded, uint64_t
     return tmd_set_error(h, TMD_ERR_ARG, "coded frame must be 16-byte aligned");
   if (coded_bytes < kHead)
     return tmd_set_error(h, TMD_ERR_ARG, "coded frame shorter than its header");
-  // handle-owned streams: each array 256-byte aligned, then the status word
-  size_t off[kFields + 1], total = 0;
-  for (int f = 0; f < kFields; f++) {
-    off[f] = total;
-    total += ((size_t)field_len(f, n_tracks, n_attached, n_unattached) * kWidth[f] + 255) & ~size_t(255);
-  }
-  off[kFields] = total;
-  total += 256;
+  const size_t total = tmd_coded_stream_bytes(n_tracks, n_attached, n_unattached);
   int rc = tmd_cuda_check(h, cudaSetDevice(h->device), "cudaSetDevice");
   if (rc != TMD_OK) return rc;
   if (total > h->coded_bytes) {
@@ -701,20 +768,8 @@ extern "C" int tmd_decode_coded_frame(tmd_handle* h, const void* coded, uint64_t
     }
     h->coded_bytes = want;
   }
-  uint8_t* b = static_cast<uint8_t*>(h->coded);
-  tmd_frame_arrays a;
-  a.n_tracks = n_tracks;
-  a.n_attached = n_attached;
-  a.n_unattached = n_unattached;
-  void** slots[kFields] = {
-      (void**)&a.qpt,      (void**)&a.row,         (void**)&a.slice,        (void**)&a.pad,
-      (void**)&a.time,     (void**)&a.ncl,         (void**)&a.qtot_a,       (void**)&a.qmax_a,
-      (void**)&a.flags_a,  (void**)&a.sigma_pad_a, (void**)&a.sigma_time_a, (void**)&a.row_diff,
-      (void**)&a.slice_leg_diff, (void**)&a.pad_res, (void**)&a.time_res,   (void**)&a.n_unatt,
-      (void**)&a.pad_diff_u, (void**)&a.time_diff_u, (void**)&a.qtot_u,     (void**)&a.qmax_u,
-      (void**)&a.flags_u,  (void**)&a.sigma_pad_u, (void**)&a.sigma_time_u};
-  for (int f = 0; f < kFields; f++) *slots[f] = b + off[f];
-  uint32_t* cstatus = reinterpret_cast<uint32_t*>(b + off[kFields]);
+  uint32_t* cstatus = nullptr;
+  const tmd_frame_arrays a = coded_arrays(h->coded, n_tracks, n_attached, n_unattached, &cstatus);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   bool order = false;  // after the previous call's use of the streams and the scratch
   if ((rc = h->order_after_previous(st, &order)) != TMD_OK) return rc;
@@ -752,17 +807,7 @@ extern "C" int tmd_decode_coded_frame(tmd_handle* h, const void* coded, uint64_t
   if (rc == TMD_OK && two)
     rc = tmd_cuda_check(h, cudaEventRecord(h->coded_late, h->aux), "cudaEventRecord");
   if (rc != TMD_OK) return rc;
-  tmd_frame_in in;
-  in.n_tracks = n_tracks;
-  in.n_attached = n_attached;
-  in.n_unattached = n_unattached;
-  in.qpt = a.qpt; in.row = a.row; in.slice = a.slice; in.pad = a.pad; in.time = a.time;
-  in.ncl = a.ncl; in.qtot_a = a.qtot_a; in.qmax_a = a.qmax_a; in.flags_a = a.flags_a;
-  in.sigma_pad_a = a.sigma_pad_a; in.sigma_time_a = a.sigma_time_a; in.row_diff = a.row_diff;
-  in.slice_leg_diff = a.slice_leg_diff; in.pad_res = a.pad_res; in.time_res = a.time_res;
-  in.n_unatt = a.n_unatt; in.pad_diff_u = a.pad_diff_u; in.time_diff_u = a.time_diff_u;
-  in.qtot_u = a.qtot_u; in.qmax_u = a.qmax_u; in.flags_u = a.flags_u;
-  in.sigma_pad_u = a.sigma_pad_u; in.sigma_time_u = a.sigma_time_u;
+  const tmd_frame_in in = frame_of(a);
   // the decode chain waits for the later streams before its record scatter
   // and unattached decode
   h->late_inputs = two ? h->coded_late : nullptr;
