@@ -252,6 +252,9 @@ extern "C" int tmd_create(const tmd_config* cfg, tmd_handle** out) {
       (rc = tmd_cuda_check(h, cudaEventCreateWithFlags(&h->scratch_done, cudaEventDisableTiming),
                            "event")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_count_rank(), "smem attribute")) != TMD_OK ||
+      (rc = tmd_cuda_check(h, cudaFuncSetAttribute(k_track_prep,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   kTrackPrepSmem), "smem attribute")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_rans_decode(), "smem attribute")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_global_xyz(&h->occ_xyz), "global transform")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_unatt_encode(&h->occ_ue), "unattached encoder")) != TMD_OK ||
@@ -554,7 +557,7 @@ int tmd_enqueue(tmd_handle* h, uint32_t nf, const tmd_frame_in* in, const tmd_fr
     most_tiles = std::max(most_tiles, fd[f].n_tiles);
   }
   if (most_tracks <= (uint32_t)kPrepTracks) {
-    timed(kKTrackPrep, [&] { launch_chained(k_track_prep, dim3(nf, 2), 1024, 0, st, dframes); });
+    timed(kKTrackPrep, [&] { launch_chained(k_track_prep, dim3(nf, 2), 1024, kTrackPrepSmem, st, dframes); });
   } else {
     if (n_tblk)
       timed(kKTrackScan1, [&] { launch_chained(k_track_scan1, n_tblk, 256, 0, st, dframes, P); });

@@ -191,6 +191,7 @@ __global__ void k_frame_scan(const FrameDev* frames, PlanDev plan);
 __global__ void k_track_scan2(const FrameDev* frames, PlanDev plan);
 // The same for frames of at most kPrepTracks tracks (grid: frames x 2).
 constexpr int kPrepTracks = 16384;
+constexpr int kTrackPrepSmem = kPrepTracks * 2;
 __global__ void k_track_prep(const FrameDev* frames);
 // Tile histograms and stable ranks of the attached clusters from their keys
 // (grid: ranking tiles of all frames).

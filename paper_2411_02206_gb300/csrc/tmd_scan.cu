@@ -152,32 +152,62 @@ __global__ void __launch_bounds__(256) k_track_scan1(const FrameDev* frames, Pla
     if (hist[i]) atomicAdd(&F.len_cursor[i], hist[i]);
 }
 
-// Starts of the unattached bins (six consecutive bins per thread, one scan),
-// their total checked, and the attached counts per bin cleared; one block of
-// 1024 threads.
-__device__ __forceinline__ void unatt_bins(const FrameDev& F) {
+// Exclusive scan of one value per bin (value(b), put(b, prefix)) by a block of
+// 1024 threads; returns the total.  Values and prefixes pass through shared
+// memory so that neighbouring lanes read and write neighbouring bins: with six
+// consecutive bins per thread in global memory a block made 3400 L1 requests,
+// which one SM takes 6.6 k cycles for.
+template <class Value, class Put>
+__device__ __forceinline__ uint32_t scan_bins(Value value, Put put) {
   constexpr int Q = (kNBin + 1023) / 1024;
+  static_assert(kNBin % Q == 0, "a thread has all its bins or none");
+  __shared__ uint32_t s_bin[kNBin];
   const uint32_t tid = threadIdx.x, b0 = tid * Q;
   uint32_t v[Q], sum = 0, tot;
 #pragma unroll
+  for (int q = 0; q < Q; q++)
+    if (tid + 1024 * q < (uint32_t)kNBin) v[q] = value(tid + 1024 * q);
+#pragma unroll
+  for (int q = 0; q < Q; q++)
+    if (tid + 1024 * q < (uint32_t)kNBin) s_bin[tid + 1024 * q] = v[q];
+  __syncthreads();
+  const bool mine = b0 < (uint32_t)kNBin;
+#pragma unroll
   for (int q = 0; q < Q; q++) {
-    v[q] = b0 + q < (uint32_t)kNBin ? F.n_unatt_bin[b0 + q] : 0u;
+    v[q] = mine ? s_bin[b0 + q] : 0u;
     sum += v[q];
   }
   uint32_t run = block_excl_scan<1024>(sum, tot);
 #pragma unroll
   for (int q = 0; q < Q; q++) {
-    if (b0 + q < (uint32_t)kNBin) F.unatt_start[b0 + q] = run;
+    if (mine) s_bin[b0 + q] = run;
     run += v[q];
   }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < Q; q++)
+    if (tid + 1024 * q < (uint32_t)kNBin) put(tid + 1024 * q, s_bin[tid + 1024 * q]);
+  return tot;
+}
+
+// Starts of the unattached bins, their total checked, and the attached counts
+// per bin cleared; one block of 1024 threads.
+__device__ __forceinline__ void unatt_bins(const FrameDev& F) {
+  const uint32_t tid = threadIdx.x;
+  const uint32_t* __restrict__ cnt = F.n_unatt_bin;
+  uint32_t* __restrict__ start = F.unatt_start;
+  uint32_t* __restrict__ att = F.att_count;
+  // attached counts: summed into by k_count_rank or k_group_sum (an encoding
+  // call has none)
+  const uint32_t tot = scan_bins([&](uint32_t b) { return cnt[b]; },
+                                 [&](uint32_t b, uint32_t v) {
+                                   start[b] = v;
+                                   if (att) att[b] = 0u;
+                                 });
   if (tid == 0) {
-    F.unatt_start[kNBin] = tot;
+    start[kNBin] = tot;
     if (tot != F.n_unatt) atomicOr(F.status, kStCount);
   }
-  // attached counts per bin: summed into by k_count_rank or k_group_sum (an
-  // encoding call has none)
-  if (F.att_count)
-    for (uint32_t b = tid; b < (uint32_t)kNBin; b += 1024) F.att_count[b] = 0u;
 }
 
 // Per frame: offsets of the track blocks, decode-order bucket offsets (longest
@@ -254,10 +284,14 @@ __global__ void __launch_bounds__(256) k_track_scan2(const FrameDev* frames, Pla
 
 // The whole track preparation of frames of at most kPrepTracks tracks in one
 // launch, two blocks per frame (tracks; unattached bins): a call of small
-// frames is a chain of latencies, and the three kernels above take 25 us
-// for 2000 tracks where this one takes 8 us.
+// frames is a chain of latencies, and the three kernels above take 25 us for 2000
+// tracks where this one takes 8 us (28 and 17 us for 11 111 tracks).
 __global__ void __launch_bounds__(1024) k_track_prep(const FrameDev* frames) {
   __shared__ uint32_t s_cur[kLenBuckets];
+  // lengths, then the order, then track starts by halves: global memory is read
+  // and written by neighbouring lanes at neighbouring tracks (see scan_bins)
+  extern __shared__ __align__(16) uint32_t s_dyn[];
+  uint16_t* s_len = reinterpret_cast<uint16_t*>(s_dyn);  // kPrepTracks
   chain_wait();
   const FrameDev& F = frames[blockIdx.x];
   if (blockIdx.y == 1) {
@@ -270,6 +304,9 @@ __global__ void __launch_bounds__(1024) k_track_prep(const FrameDev* frames) {
   const uint16_t* __restrict__ ncl = F.ncl;
   static_assert(kLenBuckets == 1024, "one bucket per thread");
   s_cur[tid] = 0u;
+#pragma unroll
+  for (int k = 0; k < E; k++)
+    if (tid + 1024 * k < nt) s_len[tid + 1024 * k] = ncl[tid + 1024 * k];
   __syncthreads();
   uint32_t n[E], sum = 0, tot;
   bool zero = false;
@@ -277,7 +314,7 @@ __global__ void __launch_bounds__(1024) k_track_prep(const FrameDev* frames) {
   for (int k = 0; k < E; k++) {
     const uint32_t t = tid * per + k;
     const bool in = (uint32_t)k < per && t < nt;
-    n[k] = in ? (uint32_t)ncl[t] : 0u;
+    n[k] = in ? (uint32_t)s_len[t] : 0u;
     sum += n[k];
     zero |= in && n[k] == 0;
     if (in) atomicAdd(&s_cur[min(n[k], (uint32_t)kLenBuckets - 1)], 1u);
@@ -291,19 +328,35 @@ __global__ void __launch_bounds__(1024) k_track_prep(const FrameDev* frames) {
   const uint32_t b = kLenBuckets - 1 - tid, v = s_cur[b];
   const uint32_t e = block_excl_scan<1024>(v, tot);
   s_cur[b] = e;
-  __syncthreads();
-  uint32_t* __restrict__ track_start = F.track_start;
-  uint32_t* __restrict__ order = F.order;
+  __syncthreads();  // also: every length is in registers
 #pragma unroll
   for (int k = 0; k < E; k++) {
     const uint32_t t = tid * per + k;
-    if ((uint32_t)k < per && t < nt) {
-      track_start[t] = start;
-      order[atomicAdd(&s_cur[min(n[k], (uint32_t)kLenBuckets - 1)], 1u)] = t;
-      start += n[k];
-      if (t == nt - 1) track_start[nt] = start;
-    }
+    if ((uint32_t)k < per && t < nt)
+      s_len[atomicAdd(&s_cur[min(n[k], (uint32_t)kLenBuckets - 1)], 1u)] = (uint16_t)t;
   }
+  __syncthreads();
+  uint32_t* __restrict__ order = F.order;
+#pragma unroll
+  for (int k = 0; k < E; k++)
+    if (tid + 1024 * k < nt) order[tid + 1024 * k] = s_len[tid + 1024 * k];
+  uint32_t* __restrict__ track_start = F.track_start;
+  constexpr uint32_t H = kPrepTracks / 2;
+  for (uint32_t h = 0; h < nt; h += H) {
+    __syncthreads();
+    uint32_t at = start;
+#pragma unroll
+    for (int k = 0; k < E; k++) {
+      const uint32_t t = tid * per + k;
+      if ((uint32_t)k < per && t < nt) {
+        if (t >= h && t < h + H) s_dyn[t - h] = at;
+        at += n[k];
+      }
+    }
+    __syncthreads();
+    for (uint32_t t = h + tid; t < nt && t < h + H; t += 1024) track_start[t] = s_dyn[t - h];
+  }
+  if (tid == 0) track_start[nt] = F.n_att;
 }
 
 // Sum of the tile histograms over groups of kGroup tiles, per bin; the group
@@ -329,25 +382,14 @@ __global__ void __launch_bounds__(kBinBlk) k_group_sum(const FrameDev* frames, P
 }
 
 // rowStart = exclusive scan of attached + unattached counts per bin, one block
-// of 1024 threads per frame, kBinPerThread consecutive bins per thread.
-constexpr int kBinPerThread = (kNBin + 1023) / 1024;
+// of 1024 threads per frame.
 __device__ __forceinline__ void row_start_scan(const FrameDev& F) {
-  uint32_t v[kBinPerThread], sum = 0, tot;
-  const uint32_t b0 = threadIdx.x * kBinPerThread;
-#pragma unroll
-  for (int q = 0; q < kBinPerThread; q++) {
-    const uint32_t b = b0 + q;
-    v[q] = b < (uint32_t)kNBin ? F.att_count[b] + F.n_unatt_bin[b] : 0u;
-    sum += v[q];
-  }
-  uint32_t run = block_excl_scan<1024>(sum, tot);
-#pragma unroll
-  for (int q = 0; q < kBinPerThread; q++) {
-    const uint32_t b = b0 + q;
-    if (b < (uint32_t)kNBin) F.row_start[b] = run;
-    run += v[q];
-  }
-  if (threadIdx.x == 0) F.row_start[kNBin] = tot;
+  const uint32_t* __restrict__ att = F.att_count;
+  const uint32_t* __restrict__ un = F.n_unatt_bin;
+  uint32_t* __restrict__ rs = F.row_start;
+  const uint32_t tot = scan_bins([&](uint32_t b) { return att[b] + un[b]; },
+                                 [&](uint32_t b, uint32_t v) { rs[b] = v; });
+  if (threadIdx.x == 0) rs[kNBin] = tot;
 }
 
 // Per frame: rowStart (the attached counts are there).

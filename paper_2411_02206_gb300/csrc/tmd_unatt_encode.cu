@@ -166,34 +166,59 @@ __device__ __forceinline__ uint32_t ue_scan(uint32_t v, uint32_t& tot) {
   return off + x - v;
 }
 
-// One block: output positions of the bins, and which kernel sorts each.
+// One block: output positions of the bins, and which kernel sorts each.  Bins
+// are read and written by neighbouring lanes at neighbouring bins, the scan over
+// consecutive bins goes through shared memory.
 __global__ void __launch_bounds__(1024) k_ue_plan(UeArgs a, UePlan* plan, UeCtl* ctl) {
-  chain_wait();
   constexpr int Q = (kNBin + 1023) / 1024;
-  const uint32_t b0 = threadIdx.x * Q;
-  uint32_t v[Q], sum = 0, tot;
+  static_assert(kNBin % Q == 0, "a thread has all its bins or none");
+  __shared__ uint32_t s_bin[kNBin];
+  __shared__ uint32_t s_block, s_big, s_general;
+  chain_wait();
+  const uint32_t tid = threadIdx.x, b0 = tid * Q;
+  uint32_t n[Q], v[Q], sum = 0, tot;
+#pragma unroll
+  for (int q = 0; q < Q; q++)
+    n[q] = tid + 1024 * q < (uint32_t)kNBin ? a.n_unatt[tid + 1024 * q] : 0u;
+#pragma unroll
+  for (int q = 0; q < Q; q++)
+    if (tid + 1024 * q < (uint32_t)kNBin) s_bin[tid + 1024 * q] = n[q];
+  if (tid == 0) s_block = s_big = s_general = 0u;
+  __syncthreads();
+  const bool mine = b0 < (uint32_t)kNBin;
 #pragma unroll
   for (int q = 0; q < Q; q++) {
-    v[q] = b0 + q < (uint32_t)kNBin ? a.n_unatt[b0 + q] : 0u;
+    v[q] = mine ? s_bin[b0 + q] : 0u;
     sum += v[q];
   }
   uint32_t run = ue_scan<1024>(sum, tot);
 #pragma unroll
   for (int q = 0; q < Q; q++) {
-    const uint32_t b = b0 + q;
-    if (b >= (uint32_t)kNBin) break;
-    plan->start[b] = plan->cursor[b] = run;
+    if (mine) s_bin[b0 + q] = run;
     run += v[q];
-    if (v[q] > kUeBigMax) {
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < Q; q++) {
+    const uint32_t b = tid + 1024 * q;
+    if (b >= (uint32_t)kNBin) break;
+    plan->start[b] = plan->cursor[b] = s_bin[b];
+    if (n[q] > kUeBigMax) {
       ctl->general[b] = 1u;
-      atomicAdd(&ctl->n_general, 1u);
-    } else if (v[q] > kUeBlockMax) {
-      plan->big[atomicAdd(&ctl->n_big, 1u)] = b;
-    } else if (v[q] > kUeWarpMax) {
-      plan->block[atomicAdd(&ctl->n_block, 1u)] = b;
+      atomicAdd(&s_general, 1u);
+    } else if (n[q] > kUeBlockMax) {
+      plan->big[atomicAdd(&s_big, 1u)] = b;
+    } else if (n[q] > kUeWarpMax) {
+      plan->block[atomicAdd(&s_block, 1u)] = b;
     }
   }
-  if (threadIdx.x == 0) plan->start[kNBin] = tot;
+  __syncthreads();
+  if (tid == 0) {
+    plan->start[kNBin] = tot;
+    ctl->n_general = s_general;
+    ctl->n_block = s_block;
+    ctl->n_big = s_big;
+  }
 }
 
 // Records to their bins.  A block counts its clusters per bin in shared memory
