@@ -81,7 +81,9 @@ typedef struct tmd_config {
  *   per bin:                         5472
  *   per unattached cluster:          n_unattached     (sum of n_unatt)
  * pad_diff_u and time_diff_u must be 16-byte aligned; other arrays need their
- * natural alignment.  A pointer whose length is 0 may be NULL. */
+ * natural alignment.  A pointer whose length is 0 may be NULL.  The kernels read
+ * the residual streams (and the encoder its truth) in aligned 16-byte pieces:
+ * bytes beside an array's ends in the same 16 bytes may be read, never used. */
 typedef struct tmd_frame_in {
   uint32_t n_tracks, n_attached, n_unattached;
   /* per track: q/pT code (q/pT = (code - 127.5) * 5/64 (GeV/c)^-1) and the
