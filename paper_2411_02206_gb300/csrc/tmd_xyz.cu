@@ -212,9 +212,9 @@ __global__ void __launch_bounds__(kXyzThreads) k_global_xyz_tiles(
         ox[k] = o.x; oy[k] = o.y; oz[k] = o.z;
       }
     }
-    *reinterpret_cast<float4*>(X + i0) = make_float4(ox[0], ox[1], ox[2], ox[3]);
-    *reinterpret_cast<float4*>(Y + i0) = make_float4(oy[0], oy[1], oy[2], oy[3]);
-    *reinterpret_cast<float4*>(Z + i0) = make_float4(oz[0], oz[1], oz[2], oz[3]);
+    __stcs(reinterpret_cast<float4*>(X + i0), make_float4(ox[0], ox[1], ox[2], ox[3]));
+    __stcs(reinterpret_cast<float4*>(Y + i0), make_float4(oy[0], oy[1], oy[2], oy[3]));
+    __stcs(reinterpret_cast<float4*>(Z + i0), make_float4(oz[0], oz[1], oz[2], oz[3]));
     stage = (stage + 1) % kTileStages;
   }
 }
@@ -232,8 +232,9 @@ cudaError_t prepare_global_xyz(int* blocks_per_sm) {
 }
 
 // Lists of kTilesFrom records and more go through the tiles (several tiles per
-// resident block), their last partial tile through the plain kernel: 240 us
-// against 266 us for 57.8 M records, 85 and 77 % of the copy bandwidth.
+// resident block), their last partial tile through the plain kernel: 237 us
+// against 266 us for 57.8 M records, 86 and 77 % of the copy bandwidth (240 us
+// without the streaming hint on the stores).
 static cudaError_t launch_global_xyz(const uint8_t* native, const uint32_t* row_start, uint32_t n,
                                      float* x, float* y, float* z, uint32_t blocks,
                                      cudaStream_t st) {
