@@ -364,7 +364,7 @@ int tmd_release(tmd_handle* h, uint64_t req_id);
  *                          the others (0), on a second stream from the start (1),
  *                          or on a second stream once the streams the track
  *                          decoder reads are done, beside the track decoder (2;
- *                          small frames from the start)
+ *                          small and very large frames from the start)
  * Defaults of a new handle: decode_variant 0, scatter_variant 1, unatt_variant 1,
  * overlap 2, decode_blocks_per_sm 0, unatt_blocks_per_sm 1, rans_overlap 1,
  * coded_overlap 2 (unless its autotune cache holds other values).

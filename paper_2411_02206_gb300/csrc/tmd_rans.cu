@@ -790,12 +790,15 @@ extern "C" int tmd_decode_coded_frame(tmd_handle* h, const void* coded, uint64_t
                          (1u << 11) | (1u << 12) | (1u << 13) | (1u << 14) | (1u << 15);
   const uint32_t later = ((1u << kFields) - 1u) & ~first;
   // coded_overlap 1: the later streams start at once beside the first ones;
-  // 2: they start when the first ones are done (beside the track decoder only),
-  // unless the frame is so small (up to 8 chunks per SM) that both leave the
-  // GPU's issue slots mostly idle: then at once
+  // 2: by the frame's chunks.  Up to 24 per SM both sets leave issue slots idle,
+  // and beyond 128 the second fills the waves of the first: at once (pp-like
+  // frame of 3.6 M clusters 274 -> 228 us, full frame 1850 -> 1817 us); in between
+  // they start when the first are done, beside the track decoder only (quarter
+  // frame 525 against 529 us)
   const bool two = h->tune_coded_overlap && h->aux && h->fork && h->coded_late;
-  const bool at_once = two && (h->tune_coded_overlap == 1 ||
-                               job_warps(a, first | later) <= 8u * (uint32_t)h->sms);
+  const uint32_t chunks = job_warps(a, first | later), sms = (uint32_t)h->sms;
+  const bool at_once =
+      two && (h->tune_coded_overlap == 1 || chunks <= 24 * sms || chunks > 128 * sms);
   if (at_once) {
     rc = tmd_cuda_check(h, cudaEventRecord(h->fork, st), "cudaEventRecord");
     if (rc == TMD_OK) rc = tmd_cuda_check(h, cudaStreamWaitEvent(h->aux, h->fork, 0), "cudaStreamWaitEvent");
