@@ -262,7 +262,9 @@ int tmd_track_trace(tmd_handle* h, const tmd_frame_in* in, uint32_t n, const uin
                     float* state, void* stream);
 
 /* Track-model encoding of the attached clusters (the synchronous side of
- * Sec. 4), device buffers, asynchronous on `stream`. */
+ * Sec. 4), device buffers, asynchronous on `stream`.  Errors: TMD_ERR_ARG (a
+ * null pointer, or an array of entries not aligned to its element size;
+ * n_attached < n_tracks), TMD_ERR_NOMEM, TMD_ERR_CUDA. */
 int tmd_encode_tracks(tmd_handle* h, const tmd_truth_in* in, const tmd_track_out* out,
                       void* stream);
 

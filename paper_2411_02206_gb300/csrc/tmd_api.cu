@@ -718,5 +718,12 @@ extern "C" int tmd_encode_tracks(tmd_handle* h, const tmd_truth_in* in, const tm
     if (na && !p) return tmd_set_error(h, TMD_ERR_ARG, "per-cluster array is NULL");
   for (const void* p : need_d)
     if (na > nt && !p) return tmd_set_error(h, TMD_ERR_ARG, "residual array is NULL");
+  // an odd address would be read as the element before it (the staged windows count in elements)
+  if ((nt && (misaligned(in->ncl, 2) || misaligned(out->pad, 2) || misaligned(out->time, 4) ||
+              misaligned(out->ncl, 2))) ||
+      (na && (misaligned(in->pad, 2) || misaligned(in->time, 4))) ||
+      (na > nt && (misaligned(out->pad_res, 2) || misaligned(out->time_res, 4))) ||
+      misaligned(out->status, 4))
+    return tmd_set_error(h, TMD_ERR_ARG, "array not aligned to its element size");
   return tmd_launch(h, 1, nullptr, nullptr, in, out, static_cast<cudaStream_t>(stream));
 }
