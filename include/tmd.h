@@ -529,9 +529,11 @@ typedef struct tmd_coded_frame {
  * form in which the paper's compressed time frames cross the host link
  * (Sec. 4, Fig. 2): frame i's coded bytes go up in one copy on a copy stream
  * while earlier frames are entropy-decoded on a stream of the handle, one frame
- * ahead of the track-model decoding on `stream`, into two handle-owned sets of
- * streams (tuning key coded_overlap 0, a single frame, or no memory for two
- * sets: on `stream`, as by tmd_decode_coded_frame), and their results come back
+ * ahead of the track-model decoding on `stream`, into the handle's set of
+ * streams and a second one in turn (tuning key coded_overlap 0, a single frame,
+ * or no memory for the second set beside the decoding scratch: on `stream`, as
+ * by tmd_decode_coded_frame; the second set is kept for later calls and given
+ * back when another allocation of the handle needs its room), and their results come back
  * to out[] on a second copy stream, through three handle-owned device slots.
  * Synchronous on return; results equal those of tmd_decode_coded_frame.
  * Errors: TMD_ERR_ARG (null pointer, n_attached < n_tracks, bytes <

@@ -149,6 +149,24 @@ int tmd_handle::mark_scratch_done(cudaStream_t st, bool order) {
   return TMD_OK;
 }
 
+bool tmd_handle::give_back_streams() {
+  if (!ent_buf) return false;
+  cudaDeviceSynchronize();
+  cudaFree(ent_buf);
+  ent_buf = nullptr;
+  ent_bytes = 0;
+  return true;
+}
+
+bool tmd_handle::device_alloc(void** p, size_t bytes) {
+  if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  if (!ent_active && give_back_streams() && cudaMalloc(p, bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  *p = nullptr;
+  return false;
+}
+
 int tmd_handle::ensure_scratch(size_t bytes) {
   if (bytes <= scratch_bytes) return TMD_OK;
   tmd_handle* h = this;
@@ -159,11 +177,8 @@ int tmd_handle::ensure_scratch(size_t bytes) {
     scratch_bytes = 0;
   }
   const size_t want = align_up(bytes + bytes / 8, 1 << 20);
-  if (cudaMalloc(&scratch, want) != cudaSuccess) {
-    cudaGetLastError();
-    scratch = nullptr;
+  if (!device_alloc(&scratch, want))
     return tmd_set_error(h, TMD_ERR_NOMEM, "cudaMalloc of %zu bytes of scratch failed", want);
-  }
   scratch_bytes = want;
   return TMD_OK;
 }
@@ -181,7 +196,7 @@ int tmd_handle::acquire_slot(size_t bytes, int& slot) {
     s.dev = nullptr;
     s.bytes = 0;
     const size_t want = align_up(bytes, 4096);
-    if (cudaMallocHost(&s.host, want) != cudaSuccess || cudaMalloc(&s.dev, want) != cudaSuccess) {
+    if (cudaMallocHost(&s.host, want) != cudaSuccess || !device_alloc(&s.dev, want)) {
       cudaGetLastError();
       return tmd_set_error(h, TMD_ERR_NOMEM, "launch record allocation failed");
     }
@@ -210,11 +225,10 @@ tmd_handle::~tmd_handle() {
   if (h2d) cudaStreamSynchronize(h2d), cudaStreamDestroy(h2d);
   if (d2h) cudaStreamSynchronize(d2h), cudaStreamDestroy(d2h);
   if (ent) cudaStreamSynchronize(ent), cudaStreamDestroy(ent);
-  for (int b = 0; b < 2; b++) {
-    if (ent_buf[b]) cudaFree(ent_buf[b]);
+  if (ent_buf) cudaFree(ent_buf);
+  for (int b = 0; b < 2; b++)
     for (cudaEvent_t e : {ent_done[b], ent_free[b]})
       if (e) cudaEventDestroy(e);
-  }
   for (int s = 0; s < kPipeSlots; s++) {
     if (pipe_buf[s]) cudaFree(pipe_buf[s]);
     for (cudaEvent_t e : {pipe_in[s], pipe_dec[s], pipe_out[s]})

@@ -94,10 +94,12 @@ struct tmd_handle {
   size_t pipe_bytes[kPipeSlots] = {};
   cudaEvent_t pipe_in[kPipeSlots] = {}, pipe_dec[kPipeSlots] = {}, pipe_out[kPipeSlots] = {};
   // coded frames: entropy decoding one frame ahead of the decode chain, into
-  // two sets of streams in turn
+  // `coded` and this second set of streams in turn.  The second set is given
+  // back when another allocation of the handle finds no room (device_alloc).
   cudaStream_t ent = nullptr;
-  void* ent_buf[2] = {};
-  size_t ent_bytes[2] = {};
+  void* ent_buf = nullptr;
+  size_t ent_bytes = 0;
+  bool ent_active = false;  // a pipeline is using the second set
   cudaEvent_t ent_done[2] = {}, ent_free[2] = {};
 
   // Calls share the scratch (and the coded-frame streams): a call on any
@@ -108,6 +110,10 @@ struct tmd_handle {
   bool scratch_busy = false;
   int order_after_previous(cudaStream_t st, bool* order);
   int mark_scratch_done(cudaStream_t st, bool order);
+  // cudaMalloc; where it fails, again without the second set of streams.
+  bool device_alloc(void** p, size_t bytes);
+  // Frees the second set of streams; true if there was one.
+  bool give_back_streams();
   int ensure_scratch(size_t bytes);
   int acquire_slot(size_t bytes, int& slot);
   ~tmd_handle();
@@ -156,6 +162,8 @@ int tmd_enqueue(tmd_handle* h, uint32_t nf, const tmd_frame_in* in, const tmd_fr
 // The two halves of tmd_decode_coded_frame on a caller's buffer of
 // tmd_coded_stream_bytes: entropy decoding into it, and the decode chain from it.
 size_t tmd_coded_stream_bytes(uint32_t n_tracks, uint32_t n_attached, uint32_t n_unattached);
+// Room for streams of that many bytes in h->coded.
+int tmd_coded_reserve(tmd_handle* h, size_t bytes);
 int tmd_coded_entropy(tmd_handle* h, const tmd_coded_frame* in, const void* coded, void* streams,
                       cudaStream_t st);
 int tmd_coded_chain(tmd_handle* h, const tmd_coded_frame* in, void* streams,

@@ -52,8 +52,8 @@ extern "C" int tmd_batch_create(tmd_handle* h, uint32_t n, const tmd_frame_in* i
   if (!b) return tmd_set_error(h, TMD_ERR_NOMEM, "batch");
   b->h = h;
   b->n = n;
-  if (cudaMalloc(&b->scratch, scratch_bytes) != cudaSuccess ||
-      cudaMalloc(&b->dev_record, record_bytes) != cudaSuccess ||
+  if (!h->device_alloc(&b->scratch, scratch_bytes) ||
+      !h->device_alloc(&b->dev_record, record_bytes) ||
       cudaMallocHost(&b->host_record, record_bytes) != cudaSuccess) {
     cudaGetLastError();
     delete b;

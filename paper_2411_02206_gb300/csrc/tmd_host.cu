@@ -125,10 +125,8 @@ int grow(tmd_handle* h, void** buf, size_t* have, size_t need) {
   }
   *buf = nullptr;
   *have = 0;
-  if (cudaMalloc(buf, need) != cudaSuccess) {
-    cudaGetLastError();
+  if (!h->device_alloc(buf, need))
     return tmd_set_error(h, TMD_ERR_NOMEM, "staging allocation of %zu bytes failed", need);
-  }
   *have = need;
   return TMD_OK;
 }
@@ -177,26 +175,28 @@ size_t coded_slot_bytes(const tmd_coded_frame& c) {
   return up(c.bytes) + up(n * TMD_REC_BYTES) + up(4 * (TMD_NBIN + 1)) + up(4 * TMD_NBIN) + 256;
 }
 
-// Stream, events and buffers of the entropy decoding ahead, made on first use;
-// false if there is no room for two sets of streams (the frames then go through
-// the handle's one set).
+// Stream, events and buffers of the entropy decoding ahead, made on first use:
+// the handle's own set of streams and a second one.  False if there is no room
+// for both (the frames then go through the handle's one set); that is not an
+// error of the call.
 bool entropy_ahead(tmd_handle* h, uint32_t n, const tmd_coded_frame* in) {
   size_t need = 0;
   for (uint32_t i = 0; i < n; i++)
     need = std::max(need, tmd_coded_stream_bytes(in[i].n_tracks, in[i].n_attached, in[i].n_unattached));
   bool ok = h->ent || cudaStreamCreateWithFlags(&h->ent, cudaStreamNonBlocking) == cudaSuccess;
-  for (int b = 0; b < 2 && ok; b++) {
+  for (int b = 0; b < 2 && ok; b++)
     for (cudaEvent_t* e : {&h->ent_done[b], &h->ent_free[b]})
       if (ok && !*e) ok = cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
-    ok = ok && grow(h, &h->ent_buf[b], &h->ent_bytes[b], need) == TMD_OK;
-  }
+  const std::string err = h->err;
+  ok = ok && tmd_coded_reserve(h, need) == TMD_OK &&
+       grow(h, &h->ent_buf, &h->ent_bytes, need) == TMD_OK;
+  // the handle's own set is shared with tmd_decode_coded_frame on any stream
+  bool order = false;
+  ok = ok && h->order_after_previous(h->ent, &order) == TMD_OK;
   if (!ok) {
     cudaGetLastError();
-    for (int b = 0; b < 2; b++) {
-      if (h->ent_buf[b]) cudaFree(h->ent_buf[b]);
-      h->ent_buf[b] = nullptr;
-      h->ent_bytes[b] = 0;
-    }
+    h->give_back_streams();
+    h->err = err;
   }
   return ok;
 }
@@ -223,10 +223,11 @@ extern "C" int tmd_decode_coded_host_stream(tmd_handle* h, uint32_t n, const tmd
   const int slots = (int)std::min<uint32_t>(n, tmd_handle::kPipeSlots);
   for (int s = 0; s < slots; s++)
     if ((rc = grow(h, &h->pipe_buf[s], &h->pipe_bytes[s], need)) != TMD_OK) return rc;
-  const bool ahead = n > 1 && h->tune_coded_overlap != 0 && entropy_ahead(h, n, in);
+  bool ahead = n > 1 && h->tune_coded_overlap != 0 && entropy_ahead(h, n, in);
   if ((rc = tmd_cuda_check(h, cudaEventRecord(h->pipe_dec[0], comp), "event")) != TMD_OK ||
       (rc = tmd_cuda_check(h, cudaStreamWaitEvent(h->h2d, h->pipe_dec[0], 0), "wait")) != TMD_OK)
     return rc;
+  h->ent_active = ahead;
   for (uint32_t i = 0; i < n && rc == TMD_OK; i++) {
     const int s = (int)(i % slots), b = (int)(i & 1);
     const tmd_coded_frame& c = in[i];
@@ -247,21 +248,33 @@ extern "C" int tmd_decode_coded_host_stream(tmd_handle* h, uint32_t n, const tmd
       rc = tmd_cuda_check(h, cudaMemcpyAsync(p, c.data, c.bytes, cudaMemcpyHostToDevice, h->h2d),
                           "H2D copy");
     if (rc == TMD_OK) rc = tmd_cuda_check(h, cudaEventRecord(h->pipe_in[s], h->h2d), "event");
+    auto whole_frame = [&] {
+      return tmd_decode_coded_frame(h, p, c.bytes, c.n_tracks, c.n_attached, c.n_unattached, &o,
+                                    comp);
+    };
     if (ahead) {
+      void* const streams = b ? h->ent_buf : h->coded;
+      const std::string err = h->err;
       // the upload, and the chain of the frame before last on these streams
       if (rc == TMD_OK) rc = tmd_cuda_check(h, cudaStreamWaitEvent(h->ent, h->pipe_in[s], 0), "wait");
       if (rc == TMD_OK && i >= 2)
         rc = tmd_cuda_check(h, cudaStreamWaitEvent(h->ent, h->ent_free[b], 0), "wait");
-      if (rc == TMD_OK) rc = tmd_coded_entropy(h, &c, p, h->ent_buf[b], h->ent);
+      if (rc == TMD_OK) rc = tmd_coded_entropy(h, &c, p, streams, h->ent);
       if (rc == TMD_OK) rc = tmd_cuda_check(h, cudaEventRecord(h->ent_done[b], h->ent), "event");
       if (rc == TMD_OK) rc = tmd_cuda_check(h, cudaStreamWaitEvent(comp, h->ent_done[b], 0), "wait");
-      if (rc == TMD_OK) rc = tmd_coded_chain(h, &c, h->ent_buf[b], &o, comp);
+      if (rc == TMD_OK) rc = tmd_coded_chain(h, &c, streams, &o, comp);
       if (rc == TMD_OK) rc = tmd_cuda_check(h, cudaEventRecord(h->ent_free[b], comp), "event");
+      if (rc == TMD_ERR_NOMEM) {
+        // no room for the chain's scratch beside the second set: this frame
+        // and those after it without that set
+        ahead = h->ent_active = false;
+        h->give_back_streams();  // waits for the frames before
+        h->err = err;
+        rc = whole_frame();
+      }
     } else {
       if (rc == TMD_OK) rc = tmd_cuda_check(h, cudaStreamWaitEvent(comp, h->pipe_in[s], 0), "wait");
-      if (rc == TMD_OK)
-        rc = tmd_decode_coded_frame(h, p, c.bytes, c.n_tracks, c.n_attached, c.n_unattached, &o,
-                                    comp);
+      if (rc == TMD_OK) rc = whole_frame();
     }
     if (rc == TMD_OK) rc = tmd_cuda_check(h, cudaEventRecord(h->pipe_dec[s], comp), "event");
     if (rc == TMD_OK) rc = tmd_cuda_check(h, cudaStreamWaitEvent(h->d2h, h->pipe_dec[s], 0), "wait");
@@ -269,6 +282,7 @@ extern "C" int tmd_decode_coded_host_stream(tmd_handle* h, uint32_t n, const tmd
     if (rc == TMD_OK) rc = tmd_cuda_check(h, cudaEventRecord(h->pipe_out[s], h->d2h), "event");
   }
   if (ahead) cudaStreamSynchronize(h->ent);
+  h->ent_active = false;
   const int rc2 = tmd_cuda_check(h, cudaStreamSynchronize(h->d2h), "stream synchronize");
   const int rc3 = tmd_cuda_check(h, cudaStreamSynchronize(comp), "stream synchronize");
   return rc != TMD_OK ? rc : (rc2 != TMD_OK ? rc2 : rc3);

@@ -720,6 +720,23 @@ size_t tmd_coded_stream_bytes(uint32_t n_tracks, uint32_t n_attached, uint32_t n
   return total;
 }
 
+int tmd_coded_reserve(tmd_handle* h, size_t bytes) {
+  if (bytes <= h->coded_bytes) return TMD_OK;
+  if (h->coded) {
+    const int rc = tmd_cuda_check(h, cudaDeviceSynchronize(), "cudaDeviceSynchronize");
+    if (rc != TMD_OK) return rc;
+    cudaFree(h->coded);
+    h->coded = nullptr;
+    h->coded_bytes = 0;
+  }
+  const size_t want = (bytes + bytes / 8 + (1u << 20)) & ~size_t((1u << 20) - 1);
+  if (!h->device_alloc(&h->coded, want))
+    return tmd_set_error(h, TMD_ERR_NOMEM, "cudaMalloc of %zu bytes of coded-frame streams failed",
+                         want);
+  h->coded_bytes = want;
+  return TMD_OK;
+}
+
 int tmd_coded_entropy(tmd_handle* h, const tmd_coded_frame* in, const void* coded, void* streams,
                       cudaStream_t st) {
   uint32_t* status = nullptr;
@@ -754,26 +771,10 @@ extern "C" int tmd_decode_coded_frame(tmd_handle* h, const void* coded, uint64_t
     return tmd_set_error(h, TMD_ERR_ARG, "coded frame must be 16-byte aligned");
   if (coded_bytes < kHead)
     return tmd_set_error(h, TMD_ERR_ARG, "coded frame shorter than its header");
-  const size_t total = tmd_coded_stream_bytes(n_tracks, n_attached, n_unattached);
   int rc = tmd_cuda_check(h, cudaSetDevice(h->device), "cudaSetDevice");
+  if (rc == TMD_OK)
+    rc = tmd_coded_reserve(h, tmd_coded_stream_bytes(n_tracks, n_attached, n_unattached));
   if (rc != TMD_OK) return rc;
-  if (total > h->coded_bytes) {
-    if (h->coded) {
-      rc = tmd_cuda_check(h, cudaDeviceSynchronize(), "cudaDeviceSynchronize");
-      if (rc != TMD_OK) return rc;
-      cudaFree(h->coded);
-      h->coded = nullptr;
-      h->coded_bytes = 0;
-    }
-    const size_t want = (total + total / 8 + (1u << 20)) & ~size_t((1u << 20) - 1);
-    if (cudaMalloc(&h->coded, want) != cudaSuccess) {
-      cudaGetLastError();
-      h->coded = nullptr;
-      return tmd_set_error(h, TMD_ERR_NOMEM, "cudaMalloc of %zu bytes of coded-frame streams failed",
-                           want);
-    }
-    h->coded_bytes = want;
-  }
   uint32_t* cstatus = nullptr;
   const tmd_frame_arrays a = coded_arrays(h->coded, n_tracks, n_attached, n_unattached, &cstatus);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
