@@ -171,6 +171,29 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t s
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// Barrier of all blocks of a cooperative launch; arrivals starts at 0, target (of
+// each thread) too.  False if they did not all arrive within kBarrierPolls polls:
+// the caller then leaves with kStTimeout.
+constexpr uint32_t kBarrierPolls = 1u << 22;
+__device__ __forceinline__ bool grid_barrier(uint32_t* arrivals, uint32_t& target) {
+  __shared__ int s_ok;
+  target += gridDim.x;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(arrivals, 1u);
+    int ok = 0;
+    for (uint32_t i = 0; i < kBarrierPolls && !ok; i++) {
+      ok = (int32_t)(*(volatile uint32_t*)arrivals - target) >= 0;
+      if (!ok) __nanosleep(64);
+    }
+    __threadfence();
+    s_ok = ok;
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
 // Kernels (launched by tmd_api.cu).
 // Launch-record upload as a kernel parameter (no copy engine), in chunks of
 // 2 KiB or 16 KiB; bytes and zero_bytes are multiples of 16.  Also clears

@@ -50,7 +50,6 @@ constexpr uint32_t kUeBigMax = 1u << 18;  // larger bins: the general sort (a sl
                                           // its whole bin, so the work grows with the square)
 constexpr uint32_t kUeBucketMax = 64;     // clusters of a bucket that one thread may sort
 constexpr int kUeScatThreads = 512;
-constexpr uint32_t kUeSpin = 1u << 22;
 
 constexpr int kRsThreads = 256;
 constexpr int kRsPerThread = 8;
@@ -610,27 +609,6 @@ __global__ void __launch_bounds__(kUeBigThreads, 1) k_ue_sort_big(UeArgs a, cons
 // cooperative launch.  Entry: {time, index, bin << 16 | pad, 0}.
 // ---------------------------------------------------------------------------
 
-// All blocks of the (cooperative) launch; false if they did not all arrive
-// within kUeSpin polls.
-__device__ __forceinline__ bool ue_grid_barrier(uint32_t* arrivals, uint32_t& target) {
-  __shared__ int s_ok;
-  target += gridDim.x;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(arrivals, 1u);
-    int ok = 0;
-    for (uint32_t i = 0; i < kUeSpin && !ok; i++) {
-      ok = (int32_t)(*(volatile uint32_t*)arrivals - target) >= 0;
-      if (!ok) __nanosleep(64);
-    }
-    __threadfence();
-    s_ok = ok;
-  }
-  __syncthreads();
-  return s_ok != 0;
-}
-
 __device__ __forceinline__ uint32_t rs_digit(const uint4& e, int pass) {
   const uint32_t w = pass < 4 ? e.y : (pass < 6 ? e.z & 0xFFFFu : (pass < 10 ? e.x : e.z >> 16));
   const int sh = pass < 4 ? pass : (pass < 6 ? pass - 4 : (pass < 10 ? pass - 6 : pass - 10));
@@ -749,7 +727,7 @@ __global__ void __launch_bounds__(kRsThreads) k_ue_general(UeArgs a, uint4* r0, 
       r1[i] = make_uint4(r.x & 0xFFFFFFu, r.w, (lo << 16) | (r.y & 0xFFFFu), 0u);
     }
   }
-  ok = ue_grid_barrier(&ctl->barrier, target);
+  ok = grid_barrier(&ctl->barrier, target);
   const uint32_t n_tiles = m / kRsTile + (m % kRsTile != 0);
   uint4* src = r1;
   uint4* dst = r0;
@@ -758,7 +736,7 @@ __global__ void __launch_bounds__(kRsThreads) k_ue_general(UeArgs a, uint4* r0, 
   for (int pass = wide ? 4 : 0; pass < 12 && ok; pass++) {
     for (uint32_t t = blockIdx.x; t < n_tiles; t += gridDim.x)
       rs_upsweep(src, m, t, n_tiles, pass, counts, s_base);
-    if (!(ok = ue_grid_barrier(&ctl->barrier, target))) break;
+    if (!(ok = grid_barrier(&ctl->barrier, target))) break;
     for (uint32_t d = blockIdx.x; d < 256; d += gridDim.x) {
       uint32_t* c = counts + (size_t)d * n_tiles;
       uint32_t run = 0;
@@ -771,7 +749,7 @@ __global__ void __launch_bounds__(kRsThreads) k_ue_general(UeArgs a, uint4* r0, 
       }
       if (tid == 0) digit_tot[d] = run;
     }
-    if (!(ok = ue_grid_barrier(&ctl->barrier, target))) break;
+    if (!(ok = grid_barrier(&ctl->barrier, target))) break;
     const uint32_t v = __ldcg(digit_tot + tid);
     uint32_t tot;
     const uint32_t e = ue_scan<kRsThreads>(v, tot);
@@ -783,7 +761,7 @@ __global__ void __launch_bounds__(kRsThreads) k_ue_general(UeArgs a, uint4* r0, 
       src = dst;
       dst = x;
     }
-    ok = ue_grid_barrier(&ctl->barrier, target);
+    ok = grid_barrier(&ctl->barrier, target);
   }
   if (!ok) {
     if (tid == 0) atomicOr(a.status, kStTimeout);

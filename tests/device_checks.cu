@@ -1,5 +1,6 @@
 // Device functions of the library checked one by one (test_gpu_device_checks.py
 // builds this file and loads it).
+#include "../paper_2411_02206_gb300/csrc/tmd_internal.cuh"
 #include "../paper_2411_02206_gb300/csrc/tmd_model.cuh"
 
 using namespace tmd;
@@ -48,11 +49,27 @@ __global__ void k_sweep(unsigned long long* bad) {
     if (n[k]) atomicAdd(&bad[k], n[k]);
 }
 
+// One grid barrier of `extra` more arrivals than there are blocks: with any, its
+// wait is bounded.  out[block] = 1 passed, 2 gave up.
+__global__ void k_barrier(uint32_t* arrivals, uint32_t extra, uint32_t* out) {
+  uint32_t target = extra;
+  const bool ok = grid_barrier(arrivals, target);
+  if (threadIdx.x == 0) out[blockIdx.x] = ok ? 1u : 2u;
+}
+
 }  // namespace
 
 extern "C" int check_sweep(unsigned long long* bad) {
   k_sweep<<<1216, 256>>>(bad);
   cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  return (int)e;
+}
+
+extern "C" int check_barrier(uint32_t blocks, uint32_t extra, uint32_t* arrivals, uint32_t* out) {
+  void* args[] = {&arrivals, &extra, &out};
+  cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_barrier, dim3(blocks), dim3(64), args,
+                                              0, nullptr);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   return (int)e;
 }

@@ -1,9 +1,10 @@
 """Device functions on their own: the track model's shortcuts (reciprocals,
 quantiser, conversions) against the operations that they stand for, bit for
-bit over every operand."""
+bit over every operand, and the bounded wait of the grid barrier."""
 import ctypes
 import os
 import subprocess
+import time
 
 import pytest
 
@@ -38,3 +39,18 @@ def test_model_shortcuts_over_all_operands(checks):
     torch.cuda.synchronize()
     assert checks.check_sweep(_ptr(bad)) == 0
     assert {k: int(v) for k, v in zip(SWEEP, bad.cpu())} == dict.fromkeys(SWEEP, 0)
+
+
+@pytest.mark.parametrize("blocks, extra", [(1, 0), (5, 0), (152, 0), (1, 1), (5, 1)])
+def test_grid_barrier_passes_or_gives_up(checks, blocks, extra):
+    """All arrivals: every block passes.  One that never comes: every block
+    gives up by itself, and the device is usable afterwards."""
+    import torch
+    arrivals = torch.zeros(1, dtype=torch.int32, device="cuda:0")
+    out = torch.zeros(blocks, dtype=torch.int32, device="cuda:0")
+    torch.cuda.synchronize()
+    t0 = time.perf_counter()
+    assert checks.check_barrier(blocks, extra, _ptr(arrivals), _ptr(out)) == 0
+    assert time.perf_counter() - t0 < 30.0
+    assert out.tolist() == [2 if extra else 1] * blocks
+    assert int(arrivals.item()) == blocks
