@@ -305,7 +305,7 @@ typedef struct tmd_unatt_out {
  * time_diff_u = the cluster's pad / time minus those of the preceding
  * cluster of its bin (the first of a bin minus 0), mod 2^16 / 2^32; charges,
  * flags and sigmas in the same order; n_unatt = clusters per bin.
- * Asynchronous on `stream`; handle scratch of about 33 bytes per cluster.
+ * Asynchronous on `stream`; handle scratch of about 33 bytes per cluster and 0.6 MB.
  * *status receives TMD_STATUS_ROW if a row >= 152 or a sector >= 36 and
  * TMD_STATUS_TIMEOUT if a bounded wait inside the sort expired (outputs then
  * unspecified).  Errors: TMD_ERR_ARG (null or misaligned pointer),
