@@ -363,10 +363,8 @@ int tmd_release(tmd_handle* h, uint64_t req_id);
  *                          entropy-decoded in one launch)
  *   "coded_overlap"  0..2  tmd_decode_coded_frame: the attached charges and the
  *                          unattached streams entropy-decoded on `stream` after
- *                          the others (0), on a second stream from the start (1),
- *                          or on a second stream once the streams the track
- *                          decoder reads are done, beside the track decoder (2;
- *                          small and very large frames from the start)
+ *                          the others (0), or on a second stream from the start
+ *                          (1, 2)
  * Defaults of a new handle: decode_variant 0, scatter_variant 1, unatt_variant 1,
  * overlap 2, decode_blocks_per_sm 0, unatt_blocks_per_sm 1, rans_overlap 1,
  * coded_overlap 2 (unless its autotune cache holds other values).

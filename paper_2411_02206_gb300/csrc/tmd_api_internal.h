@@ -66,7 +66,7 @@ struct tmd_handle {
   int tune_unatt_bps = 1;        // unattached-decode blocks per SM (0: as many as fit)
   int tune_rans_overlap = 1;      // no effect: all widths are entropy-decoded in one launch
   int tune_coded_overlap = 2;    // coded frames: charges and unattached streams entropy-
-                                 // decoded on the second stream beside the track decoder
+                                 // decoded on the second stream (1, 2) or after the others (0)
   cudaEvent_t coded_late = nullptr;   // recorded after those streams are decoded
   cudaEvent_t late_inputs = nullptr;  // set for the chain of a coded frame
   uint64_t mem_budget = 0;

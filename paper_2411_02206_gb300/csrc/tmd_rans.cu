@@ -19,10 +19,10 @@
 // widths share a launch, the widest first: a lane's chain of 256 to 1024
 // dependent symbols takes tens of microseconds whatever the frame's size, and
 // launches of one width after another add those up.
-// tmd_decode_coded_frame entropy-decodes the streams the track decoder and the
-// ranking read first and the attached charges and unattached streams on the
-// second stream while the track decoder runs; the decode chain waits for them
-// before its record scatter and unattached decode.
+// tmd_decode_coded_frame entropy-decodes the streams that the track decoder and the
+// ranking read on the caller's stream and the attached charges and unattached streams
+// beside them on the second stream; the decode chain waits for those before its
+// record scatter and unattached decode.
 #include <algorithm>
 #include <atomic>
 #include <cstring>
@@ -783,24 +783,20 @@ extern "C" int tmd_decode_coded_frame(tmd_handle* h, const void* coded, uint64_t
   rc = tmd_cuda_check(h, cudaMemsetAsync(cstatus, 0, 4, st), "cudaMemsetAsync");
   if (rc != TMD_OK) return rc;
   // The streams the track decoder and the ranking read (headers, differences,
-  // residuals, the per-bin unattached counts) are entropy-decoded first on
-  // `stream`; the charges of the attached clusters and the unattached streams,
-  // needed only by the record scatter and the unattached decode, on the
-  // handle's second stream while the track decoder runs.
+  // residuals, the per-bin unattached counts) are entropy-decoded on `stream`; the
+  // charges of the attached clusters and the unattached streams, needed only by
+  // the record scatter and the unattached decode, on the handle's second stream.
   const uint32_t first = (1u << 0) | (1u << 1) | (1u << 2) | (1u << 3) | (1u << 4) | (1u << 5) |
                          (1u << 11) | (1u << 12) | (1u << 13) | (1u << 14) | (1u << 15);
   const uint32_t later = ((1u << kFields) - 1u) & ~first;
-  // coded_overlap 1: the later streams start at once beside the first ones;
-  // 2: by the frame's chunks.  Up to 24 per SM both sets leave issue slots idle,
-  // and beyond 128 the second fills the waves of the first: at once (pp-like
-  // frame of 3.6 M clusters 274 -> 228 us, full frame 1850 -> 1817 us); in between
-  // they start when the first are done, beside the track decoder only (quarter
-  // frame 525 against 529 us)
+  // They start at once beside the first ones.  Starting when the first are done,
+  // beside the track decoder only, was the slower order in a sweep of 47 frames
+  // from 6 to 160 chunks per SM: at once takes 0.71 to 0.98 of its time for pp-like
+  // mixes up to 95 chunks per SM, 0.75 to 1.01 for stress mixes, 0.83 to 1.13 for
+  // Pb-Pb mixes (above 1.02 at 20 and 27 chunks per SM only; 0.97 on average) and
+  // between 0.95 and 1.02 for all beyond 95 (quarter Pb-Pb frame 523 against 521 us).
   const bool two = h->tune_coded_overlap && h->aux && h->fork && h->coded_late;
-  const uint32_t chunks = job_warps(a, first | later), sms = (uint32_t)h->sms;
-  const bool at_once =
-      two && (h->tune_coded_overlap == 1 || chunks <= 24 * sms || chunks > 128 * sms);
-  if (at_once) {
+  if (two) {
     rc = tmd_cuda_check(h, cudaEventRecord(h->fork, st), "cudaEventRecord");
     if (rc == TMD_OK) rc = tmd_cuda_check(h, cudaStreamWaitEvent(h->aux, h->fork, 0), "cudaStreamWaitEvent");
     if (rc != TMD_OK) return rc;
@@ -808,10 +804,6 @@ extern "C" int tmd_decode_coded_frame(tmd_handle* h, const void* coded, uint64_t
   const uint8_t* c = static_cast<const uint8_t*>(coded);
   cudaStream_t late_st = two ? h->aux : st;
   rc = tmd_cuda_check(h, launch_streams(h, c, coded_bytes, a, cstatus, st, first), "k_rans_decode");
-  if (rc == TMD_OK && two && !at_once) {
-    rc = tmd_cuda_check(h, cudaEventRecord(h->fork, st), "cudaEventRecord");
-    if (rc == TMD_OK) rc = tmd_cuda_check(h, cudaStreamWaitEvent(h->aux, h->fork, 0), "cudaStreamWaitEvent");
-  }
   if (rc == TMD_OK)
     rc = tmd_cuda_check(h, launch_streams(h, c, coded_bytes, a, cstatus, late_st, later), "k_rans_decode");
   if (rc == TMD_OK && two)
