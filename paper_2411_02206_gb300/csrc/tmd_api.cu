@@ -275,7 +275,7 @@ extern "C" int tmd_create(const tmd_config* cfg, tmd_handle** out) {
       (rc = tmd_cuda_check(h, prepare_track_decode(0, &h->occ_decode_v[0]), "occupancy")) != TMD_OK ||
       (rc = tmd_cuda_check(h, prepare_track_decode(1, &h->occ_decode_v[1]), "occupancy")) != TMD_OK ||
       (rc = tmd_cuda_check(h, occupancy_unatt_decode(&h->occ_unatt), "occupancy")) != TMD_OK ||
-      (rc = tmd_cuda_check(h, prepare_track_encode(&h->occ_encode), "occupancy")) != TMD_OK) {
+      (rc = tmd_cuda_check(h, prepare_track_encode(h->occ_encode), "occupancy")) != TMD_OK) {
     delete h;
     return rc;
   }
@@ -284,7 +284,7 @@ extern "C" int tmd_create(const tmd_config* cfg, tmd_handle** out) {
   h->occ_decode = h->occ_decode_v[h->tune_decode_variant];
   if (!h->autotune_cache.empty()) tmd_tune_load(h);
   if (h->occ_unatt < 1) h->occ_unatt = 1;
-  if (h->occ_encode < 1) h->occ_encode = 1;
+  for (int& o : h->occ_encode) o = std::max(o, 1);
   if (h->occ_ue < 1) h->occ_ue = 1;
   if (h->occ_xyz < 1) h->occ_xyz = 1;
   *out = h;
@@ -466,8 +466,11 @@ int tmd_enqueue(tmd_handle* h, uint32_t nf, const tmd_frame_in* in, const tmd_fr
   EncDev* ed = reinterpret_cast<EncDev*>(host + R.enc);
   pre_tblk[0] = pre_tile[0] = pre_grp[0] = pre_warp[0] = pre_chunk[0] = pre_kt[0] = 0;
   uint32_t* zero_bins = reinterpret_cast<uint32_t*>(zb + 256);
-  uint64_t all_tracks = 0;
-  for (uint32_t f = 0; f < nf; f++) all_tracks += encode ? tin[f].n_tracks : in[f].n_tracks;
+  uint64_t all_tracks = 0, all_attached = 0;
+  for (uint32_t f = 0; f < nf; f++) {
+    all_tracks += encode ? tin[f].n_tracks : in[f].n_tracks;
+    all_attached += encode ? tin[f].n_attached : in[f].n_attached;
+  }
   const uint32_t lanes = task_lanes(all_tracks, (uint32_t)h->sms);
   for (uint32_t f = 0; f < nf; f++) {
     FrameDev& F = fd[f];
@@ -584,12 +587,11 @@ int tmd_enqueue(tmd_handle* h, uint32_t nf, const tmd_frame_in* in, const tmd_fr
       k_track_trace<<<(trace->n + 127) / 128, 128, 0, st>>>(dframes, trace->ids, trace->n,
                                                             trace->state);
   } else if (encode) {
-    if (n_warp) {
-      const uint32_t per_block = kDecodeThreads / 32;
-      const uint32_t grid = std::min<uint32_t>((n_warp + per_block - 1) / per_block,
-                                               (uint32_t)(h->sms * h->occ_encode));
-      timed(kKTrackEncode, [&] { launch_track_encode(grid, st, denc, dframes, P, n_warp); });
-    }
+    if (n_warp)
+      timed(kKTrackEncode, [&] {
+        launch_track_encode(all_tracks, all_attached, (uint32_t)h->sms, h->occ_encode, st,
+                            denc, dframes, P, n_warp);
+      });
   } else {
     // track decode (keys, pad and time codes), per-tile counts and ranks, row
     // offsets; then the tile bases and the record scatter, with the

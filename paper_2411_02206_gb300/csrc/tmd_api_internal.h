@@ -54,7 +54,8 @@ struct tmd_handle {
   };
   int device = 0;
   int sms = 0;
-  int occ_decode = 1, occ_unatt = 1, occ_encode = 1, occ_ue = 1, occ_xyz = 1;
+  int occ_decode = 1, occ_unatt = 1, occ_ue = 1, occ_xyz = 1;
+  int occ_encode[2] = {1, 1};    // of the track encoder, and of the one for short tracks
   int occ_decode_v[2] = {1, 1};  // resident blocks per SM of the decoder variants
   // tuning parameters (launch shapes only; results never depend on them)
   int tune_decode_variant = 0;   // staging-round variant of the track decoder

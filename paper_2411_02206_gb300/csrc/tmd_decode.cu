@@ -33,6 +33,8 @@
 //
 // Encoder: the same walk with the truth as measurement; it writes the header
 // and the residual streams (the synchronous side of the method).
+#include <algorithm>
+
 #include "tmd_internal.cuh"
 
 namespace tmd {
@@ -430,10 +432,11 @@ __device__ __forceinline__ void issue_truth(uint32_t* buf, const Truth& E, uint3
 // Writes the headers and the residual streams of the attached clusters.  One
 // lane per track like the decoder, with the truth staged a round ahead and the
 // residuals leaving through shared memory: read and written directly, 13
-// unrelated sectors per lane and step, the walk took 3.25 ms for 200 k tracks
+// unrelated sectors per lane and step, the walk took 2.72 ms for 200 k tracks
 // (18 M clusters); staged it takes 0.30 ms.
 __global__ void __launch_bounds__(kDecodeThreads, 3)
-    k_track_encode(const EncDev* enc, const FrameDev* frames, PlanDev plan, uint32_t n_tasks) {
+    k_track_encode(const EncDev* enc, const FrameDev* frames, PlanDev plan, uint32_t n_tasks,
+                   uint32_t too_short) {
   constexpr int R = kEncRound, P = EncStage::kPitch;
   __shared__ RowGeo geo;
   extern __shared__ __align__(16) uint32_t s_stage[];
@@ -466,7 +469,9 @@ __global__ void __launch_bounds__(kDecodeThreads, 3)
       n = D.ncl[t];
     }
     const uint32_t dm1 = j0 - t - 1u;  // cluster k >= 1 has difference dm1 + k
-    const uint32_t rounds = (__reduce_max_sync(kFull, n) + R - 1) / R;
+    const uint32_t nmax = __reduce_max_sync(kFull, n);
+    if (nmax <= too_short) break;  // this task and those after it: k_track_encode_short
+    const uint32_t rounds = (nmax + R - 1) / R;
     uint32_t* lb0 = S.buf[0] + lane * EncStage::kLane;
     uint32_t* lb1 = S.buf[1] + lane * EncStage::kLane;
     issue_truth(S.buf[0], E, j0, min(n, (uint32_t)R), lanes);
@@ -587,10 +592,97 @@ __global__ void __launch_bounds__(kDecodeThreads, 3)
 
 constexpr int kEncodeSmem = (kDecodeThreads / 32) * (int)sizeof(EncStage);
 
-void launch_track_encode(uint32_t grid, cudaStream_t st, const EncDev* enc, const FrameDev* frames,
-                         PlanDev plan, uint32_t n_tasks) {
-  launch_chained(k_track_encode, grid, kDecodeThreads, kEncodeSmem, st, enc, frames, plan,
-                 n_tasks);
+// The same walk for tracks of up to kShortTrack clusters, read and written directly:
+// a warp's time is that of fetching its task, and what counts is warps per SM.  Tasks
+// with a longer track are left to k_track_encode.
+constexpr uint32_t kShortTrack = 4;
+constexpr int kShortThreads = 256;
+__global__ void __launch_bounds__(kShortThreads, 4)
+    k_track_encode_short(const EncDev* enc, const FrameDev* frames, PlanDev plan,
+                         uint32_t n_tasks) {
+  __shared__ RowGeo geo;
+  fill_row_geo(&geo);
+  chain_wait();
+  __syncthreads();
+  const uint32_t lane = threadIdx.x & 31, lanes = plan.lanes;
+  const FrameDev& F = frames[0];  // an encoding call has one frame
+  const EncDev& D = enc[0];
+  if (*F.status & kStCount) return;
+  const Truth E{D.row, D.sector, D.leg, D.pad, D.time};
+  for (;;) {
+    const uint32_t ticket = next_task(&plan.counters[1]);
+    if (ticket >= n_tasks) break;
+    const uint32_t idx = lane < lanes ? ticket * lanes + lane : 0xFFFFFFFFu;
+    uint32_t st = 0, t = 0, j0 = 0, n = 0, r0 = 0, s0 = 0, l0 = 0, pad = 0, time = 0;
+    uint8_t qpt = 0;
+    Track s;
+    if (idx < F.n_tracks) {
+      t = F.order[idx];
+      j0 = F.track_start[t];
+      n = D.ncl[t];
+      r0 = E.row[j0];
+      s0 = E.sector[j0];
+      l0 = E.leg[j0];
+      pad = E.pad[j0], time = E.time[j0];
+      qpt = D.qpt[t];
+    }
+    const uint32_t nmax = __reduce_max_sync(kFull, n);
+    if (nmax > kShortTrack) continue;
+    if (n > 0) {
+      if (r0 >= (uint32_t)kNRow || s0 >= (uint32_t)kNSec) st |= kStRow;
+      D.o_qpt[t] = qpt;
+      D.o_ncl[t] = (uint16_t)n;
+      D.o_row[t] = (uint8_t)r0;
+      D.o_slice[t] = (uint8_t)s0;
+      D.o_pad[t] = (uint16_t)pad;
+      D.o_time[t] = time;
+      if (n > 1) seed(&geo, s, qpt, (int)r0, s0 < (uint32_t)kNSec ? (int)s0 : kNSec - 1, pad, time);
+    }
+    for (uint32_t k = 1; k < nmax; k++) {
+      if (k >= n) continue;
+      const uint32_t d = j0 - t + k - 1, j = j0 + k;
+      const uint32_t r1 = E.row[j], s1 = E.sector[j], l1 = E.leg[j];
+      const uint32_t padq = E.pad[j], timeq = E.time[j];
+      if (r1 >= (uint32_t)kNRow || s1 >= (uint32_t)kNSec) st |= kStRow;
+      const uint32_t sld = (l1 != l0 ? (uint32_t)kNSec : 0u) + (s1 - s0 + 8u * kNSec) % kNSec;
+      D.o_row_diff[d] = (uint8_t)(r1 - r0);
+      D.o_sld[d] = (uint8_t)sld;
+      r0 = r1;
+      s0 = s1;
+      l0 = l1;
+      row_step(s, (int)r1);
+      turn_step(&geo, s, sld);
+      uint32_t ppad, ptime;
+      const float4 G = geo.row[s.row];
+      propagate_predict(G, s, ppad, ptime);
+      D.o_pad_res[d] = (uint16_t)((padq - ppad) & 0xFFFFu);
+      D.o_time_res[d] = timeq - ptime;
+      update(G, s, padq, timeq);
+    }
+    st = __reduce_or_sync(kFull, st);
+    if (st && lane == 0) atomicOr(F.status, st);
+  }
+}
+
+// Calls of up to kShortTrack clusters per track go to both kernels, the others to
+// the staged one alone.  A million tracks of 1, 2, 3, 4, 6 and 8 clusters: 96, 103, 124, 157,
+// 234 and 321 us by the short walk, 149, 173, 177, 181, 203 and 218 us staged; 300 k: 66, 70,
+// 79, 91, 110 and 136 against 86, 96, 95, 98, 100 and 106 us.  The short walk goes first: behind
+// the staged kernel, whose shared memory leaves it little L1, 4 M tracks of 4 clusters
+// take 565 instead of 454 us.
+void launch_track_encode(uint64_t n_tracks, uint64_t n_attached, uint32_t sms,
+                         const int* blocks_per_sm, cudaStream_t st, const EncDev* enc,
+                         const FrameDev* frames, PlanDev plan, uint32_t n_tasks) {
+  const bool both = n_attached <= kShortTrack * n_tracks;
+  auto grid = [&](uint32_t threads, int bps) {
+    const uint32_t per_block = threads / 32;
+    return std::min<uint32_t>((n_tasks + per_block - 1) / per_block, sms * (uint32_t)bps);
+  };
+  if (both)
+    launch_chained(k_track_encode_short, grid(kShortThreads, blocks_per_sm[1]), kShortThreads, 0, st,
+                   enc, frames, plan, n_tasks);
+  launch_chained(k_track_encode, grid(kDecodeThreads, blocks_per_sm[0]), kDecodeThreads, kEncodeSmem,
+                 st, enc, frames, plan, n_tasks, both ? kShortTrack : 0u);
 }
 
 cudaError_t prepare_track_encode(int* blocks_per_sm) {

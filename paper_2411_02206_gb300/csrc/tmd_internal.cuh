@@ -105,7 +105,8 @@ struct PlanDev {
   const uint32_t* pre_chunk;  // unattached chunks
   const uint32_t* pre_kt;     // decoder: warp tasks
   uint32_t lanes;             // tracks per warp task (task_lanes)
-  uint32_t* counters;         // [0] decode/encode task, [1] unattached ticket (zeroed)
+  uint32_t* counters;         // [0] decode/encode task, [1] unattached ticket, short
+                              // tracks of an encoding call (zeroed)
 };
 
 // Tracks per warp task of the track decoder and encoder, one lane each.  A call
@@ -250,8 +251,10 @@ void launch_unatt_decode(int variant, uint32_t grid, cudaStream_t st, const Fram
                          PlanDev plan, uint32_t n_tickets, bool chained = false);
 cudaError_t occupancy_unatt_decode(int* blocks_per_sm);
 __global__ void k_selftest_wait(const unsigned long long* never, uint32_t* status);
-void launch_track_encode(uint32_t grid, cudaStream_t st, const EncDev* enc, const FrameDev* frames,
-                         PlanDev plan, uint32_t n_tasks);
+// One frame.  blocks_per_sm: of the kernel and of the one for short tracks.
+void launch_track_encode(uint64_t n_tracks, uint64_t n_attached, uint32_t sms,
+                         const int* blocks_per_sm, cudaStream_t st, const EncDev* enc,
+                         const FrameDev* frames, PlanDev plan, uint32_t n_tasks);
 cudaError_t prepare_track_encode(int* blocks_per_sm);
 __global__ void k_track_trace(const FrameDev* frames, const uint32_t* ids, uint32_t n_ids,
                               float* state);
