@@ -686,11 +686,15 @@ void launch_track_encode(uint64_t n_tracks, uint64_t n_attached, uint32_t sms,
 }
 
 cudaError_t prepare_track_encode(int* blocks_per_sm) {
-  const cudaError_t e = cudaFuncSetAttribute(
-      k_track_encode, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncodeSmem);
-  if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_track_encode,
-                                                       kDecodeThreads, kEncodeSmem);
+  cudaError_t e = cudaFuncSetAttribute(k_track_encode, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       kEncodeSmem);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm[0], k_track_encode,
+                                                      kDecodeThreads, kEncodeSmem);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm[1], k_track_encode_short,
+                                                      kShortThreads, 0);
+  return e;
 }
 
 }  // namespace tmd
