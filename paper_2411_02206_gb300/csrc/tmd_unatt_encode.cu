@@ -76,8 +76,11 @@ struct UeCtl {
 struct UePlan {
   uint32_t start[kNBin + 1];   // first output position of every bin
   uint32_t cursor[kNBin];      // next free record of every bin during the scatter
-  uint32_t block[kNBin];             // bins
-  uint32_t big[kNBin * kUeSlices];   // bin << 8 | time slice or kUeWhole
+  uint32_t block[kNBin];       // bins
+};
+// bin << 8 | time slice or kUeWhole
+struct UeBig {
+  uint32_t item[kNBin * kUeSlices];
 };
 
 struct UeArgs {
@@ -176,8 +179,8 @@ __device__ __forceinline__ uint32_t ue_scan(uint32_t v, uint32_t& tot) {
 // One block: output positions of the bins, and which kernel sorts each.  Bins
 // are read and written by neighbouring lanes at neighbouring bins, the scan over
 // consecutive bins goes through shared memory.
-__global__ void __launch_bounds__(1024) k_ue_plan(UeArgs a, UePlan* plan, UeCtl* ctl,
-                                                  uint32_t sms) {
+__global__ void __launch_bounds__(1024) k_ue_plan(UeArgs a, UePlan* plan, UeBig* big,
+                                                  UeCtl* ctl, uint32_t sms) {
   constexpr int Q = (kNBin + 1023) / 1024;
   static_assert(kNBin % Q == 0, "a thread has all its bins or none");
   __shared__ uint32_t s_bin[kNBin];
@@ -216,7 +219,7 @@ __global__ void __launch_bounds__(1024) k_ue_plan(UeArgs a, UePlan* plan, UeCtl*
       atomicAdd(&s_general, 1u);
     } else if (n[q] > kUeBlockMax) {
       atomicAdd(&s_bins, 1u);
-      if (n[q] <= kUeSliceMean) plan->big[atomicAdd(&s_big, 1u)] = (b << 8) | kUeWhole;
+      if (n[q] <= kUeSliceMean) big->item[atomicAdd(&s_big, 1u)] = (b << 8) | kUeWhole;
       else s_sliced = 1u;
     } else if (n[q] > kUeWarpMax) {
       plan->block[atomicAdd(&s_block, 1u)] = b;
@@ -232,7 +235,7 @@ __global__ void __launch_bounds__(1024) k_ue_plan(UeArgs a, UePlan* plan, UeCtl*
       const bool whole = slices <= kUeWholeSlices && s_bins >= sms;
       const uint32_t count = whole ? 1u : slices;
       const uint32_t at = atomicAdd(&s_big, count);
-      for (uint32_t k = 0; k < count; k++) plan->big[at + k] = (b << 8) | (whole ? kUeWhole : k);
+      for (uint32_t k = 0; k < count; k++) big->item[at + k] = (b << 8) | (whole ? kUeWhole : k);
     }
     __syncthreads();
   }
@@ -591,7 +594,8 @@ __global__ void __launch_bounds__(kUeBlockThreads, 3) k_ue_sort_block(UeArgs a, 
 // whole (152 of 20 k: 146 against 158 us; 547 of 40 k: 1.03 against 1.07 ms), larger
 // ones by slices (152 of 50 k: 0.40 against 0.44 ms; 300 of 60 k: 0.90 against 1.05).
 __global__ void __launch_bounds__(kUeBigThreads, 1) k_ue_sort_big(UeArgs a, const uint4* rec,
-                                                                 const UePlan* plan, UeCtl* ctl) {
+                                                                 const UePlan* plan,
+                                                                 const UeBig* big, UeCtl* ctl) {
   chain_wait();
   constexpr int T = kUeBigThreads, E = kUeSliceCap / T;
   extern __shared__ uint64_t s_dyn[];
@@ -611,7 +615,7 @@ __global__ void __launch_bounds__(kUeBigThreads, 1) k_ue_sort_big(UeArgs a, cons
     __syncthreads();
     const uint32_t task = s_task;
     if (task >= n_list) break;
-    const uint32_t b = plan->big[task] >> 8, part = plan->big[task] & 255u;
+    const uint32_t b = big->item[task] >> 8, part = big->item[task] & 255u;
     const uint32_t s0 = plan->start[b], n = plan->start[b + 1] - s0;
     const uint4* __restrict__ r0 = rec + s0;
     uint32_t lo = 0xFFFFFFFFu, hi = 0u;
@@ -1096,8 +1100,9 @@ extern "C" int tmd_encode_unattached(tmd_handle* h, const tmd_unatt_truth_in* in
   const uint32_t n_tiles = n / kRsTile + 1;
   auto up = [](size_t x) { return (x + 255) / 256 * 256; };
   const size_t o_r0 = 0, o_r1 = up((size_t)n * 16 + 16), o_cnt = o_r1 + up((size_t)n * 16 + 16),
-               o_dig = o_cnt + up((size_t)256 * n_tiles * 4), o_ctl = o_dig + up(256 * 4),
-               o_plan = o_ctl + up(sizeof(UeCtl)), total = o_plan + up(sizeof(UePlan));
+               o_dig = o_cnt + up((size_t)256 * n_tiles * 4), o_plan = o_dig + up(256 * 4),
+               o_ctl = o_plan + up(sizeof(UePlan)), o_big = o_ctl + up(sizeof(UeCtl)),
+               total = o_big + up(sizeof(UeBig));
   if ((rc = h->ensure_scratch(total)) != TMD_OK) return rc;
   bool order = false;
   if ((rc = h->order_after_previous(st, &order)) != TMD_OK) return rc;
@@ -1108,6 +1113,7 @@ extern "C" int tmd_encode_unattached(tmd_handle* h, const tmd_unatt_truth_in* in
   uint32_t* dig = reinterpret_cast<uint32_t*>(base + o_dig);
   UePlan* plan = reinterpret_cast<UePlan*>(base + o_plan);
   UeCtl* ctl = reinterpret_cast<UeCtl*>(base + o_ctl);
+  UeBig* big = reinterpret_cast<UeBig*>(base + o_big);
   UeArgs a;
   a.n = n;
   a.row = in->row; a.sector = in->sector; a.pad = in->pad; a.time = in->time;
@@ -1122,7 +1128,7 @@ extern "C" int tmd_encode_unattached(tmd_handle* h, const tmd_unatt_truth_in* in
   k_ue_init<<<(sizeof(UeCtl) / 4 + 255) / 256, 256, 0, st>>>(a, ctl);
   if (n) {
     launch_chained(k_ue_count, std::min(2 * sms, n / 8192 + 1), 1024, 0, st, a);
-    launch_chained(k_ue_plan, 1, 1024, 0, st, a, plan, ctl, sms);
+    launch_chained(k_ue_plan, 1, 1024, 0, st, a, plan, big, ctl, sms);
     launch_chained(k_ue_scatter, n / (kUeScatThreads * 4) + (n % (kUeScatThreads * 4) != 0),
                    kUeScatThreads, 0, st, a, r0, plan, ctl);
     launch_chained(k_ue_sort_warp, (kNBin + 7) / 8, 256, 0, st, a, r0, plan, ctl);
@@ -1131,7 +1137,7 @@ extern "C" int tmd_encode_unattached(tmd_handle* h, const tmd_unatt_truth_in* in
                      kUeBlockSmem, st, a, r0, plan, ctl);
     if (n > kUeBlockMax)
       launch_chained(k_ue_sort_big, std::min(sms, n / kUeBlockMax), kUeBigThreads, kUeBigSmem, st,
-                     a, r0, plan, ctl);
+                     a, r0, plan, big, ctl);
     void* args[] = {&a, &r0, &r1, &plan, &ctl, &cnt, &dig};
     const uint32_t grid = std::min(n_tiles, sms * (uint32_t)h->occ_ue);
     rc = tmd_cuda_check(h, cudaLaunchCooperativeKernel((const void*)k_ue_general, dim3(grid),
