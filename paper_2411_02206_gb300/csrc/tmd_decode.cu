@@ -5,9 +5,10 @@
 //
 // Decoding of the attached clusters runs in three kernels:
 //
-//   k_track_decode  one lane per track, warps take 32 tracks at a time from
-//                   the length-sorted order (longest first, so lanes of a warp
-//                   run loops of similar length and the tail is short).  For
+//   k_track_decode  one lane per track, warps take up to 32 tracks at a time
+//                   (task_lanes) from the length-sorted order (longest first,
+//                   so lanes of a warp run loops of similar length and the tail
+//                   is short).  For
 //                   every cluster the lane applies the row and sector/leg
 //                   differences, propagates the model to the row, adds the
 //                   modular residuals to the quantised prediction and updates
