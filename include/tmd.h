@@ -509,8 +509,8 @@ int tmd_rans_decode(tmd_handle* h, const void* coded, uint64_t coded_bytes,
  * streams are decoded into handle-owned device memory (grown on demand) and
  * the frame is then decoded as by tmd_decode_frame into `out`, on `stream`
  * (the streams only the record scatter and the unattached decode read are
- * entropy-decoded on the handle's second stream beside the track decoder,
- * tuning key coded_overlap).  out->status receives TMD_STATUS_CODED as well as the decoder's
+ * entropy-decoded on the handle's second stream beside the others, tuning key
+ * coded_overlap).  out->status receives TMD_STATUS_CODED as well as the decoder's
  * bits.  Errors as tmd_rans_decode and tmd_decode_frame, plus TMD_ERR_NOMEM. */
 int tmd_decode_coded_frame(tmd_handle* h, const void* coded, uint64_t coded_bytes,
                            uint32_t n_tracks, uint32_t n_attached, uint32_t n_unattached,
