@@ -790,11 +790,12 @@ extern "C" int tmd_decode_coded_frame(tmd_handle* h, const void* coded, uint64_t
                          (1u << 11) | (1u << 12) | (1u << 13) | (1u << 14) | (1u << 15);
   const uint32_t later = ((1u << kFields) - 1u) & ~first;
   // They start at once beside the first ones.  Starting when the first are done,
-  // beside the track decoder only, was the slower order in a sweep of 47 frames
-  // from 6 to 160 chunks per SM: at once takes 0.71 to 0.98 of its time for pp-like
-  // mixes up to 95 chunks per SM, 0.75 to 1.01 for stress mixes, 0.83 to 1.13 for
-  // Pb-Pb mixes (above 1.02 at 20 and 27 chunks per SM only; 0.97 on average) and
-  // between 0.95 and 1.02 for all beyond 95 (quarter Pb-Pb frame 523 against 521 us).
+  // beside the track decoder only, is no faster at any size: in a sweep of five mixes
+  // at 23 sizes, at once takes 0.86 to 0.99 of its time (means over the mixes) from
+  // 18 to 80 chunks per SM and 0.97 to 1.01 from there to 136.  Single frames: 0.76 at
+  // best (pp-like, up to 28 chunks per SM), at worst 1.12 (Pb-Pb, 23 and 27, where a
+  // part of the blocks starts a second wave) and 1.035 elsewhere; the quarter Pb-Pb
+  // frame 524 against 519 us, one of 5 M clusters 285 against 329 us.
   const bool two = h->tune_coded_overlap && h->aux && h->fork && h->coded_late;
   if (two) {
     rc = tmd_cuda_check(h, cudaEventRecord(h->fork, st), "cudaEventRecord");
